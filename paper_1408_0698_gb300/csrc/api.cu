@@ -182,10 +182,10 @@ struct LoopDm {
 // mirror layer, OPD, expected images and slopes.
 struct CalibScratch {
     int gs = -1, kind = 0, geom = 0, group = 0, nv = 0, blocks_per_wfs = 0;
-    size_t opd_stride = 0, det_stride = 0;
+    size_t opd_stride = 0;
     WfsDesc *d_wfs = nullptr;        // [kMaxInstances]
     InstDesc *d_inst = nullptr;      // [n_dm][kMaxInstances]: a mirror as the only layer
-    float *opd = nullptr, *E = nullptr, *slopes = nullptr, *layers = nullptr;
+    float *opd = nullptr, *slopes = nullptr, *layers = nullptr;
     int *work = nullptr;             // ticket pairs: projection, spot kernel
     int cur_dm = -1;                 // mirror whose windows the layer buffers hold
 };
@@ -552,7 +552,7 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
     dyn.opd = (st && st->opd) ? st->opd : h->d_opd;
     dyn.slopes = slopes;
     dyn.st_I = st ? st->intensity : nullptr;
-    dyn.st_E = (st && st->expected) ? st->expected : h->d_E;  // the split noise pass reads E back
+    dyn.st_E = st ? st->expected : nullptr;
     dyn.st_C = st ? st->counts : nullptr;
     dyn.t = t;
     dyn.noise = h->noise;
@@ -612,9 +612,10 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         sa.n_inst = 1;
         sa.work = h->d_work + 2 * (&G - h->groups.data());
         sa.project = project_mode;
-        sa.split_noise = splits_noise(G.kind, sa.N, sa.nd) ? 1 : 0;
+        sa.split_noise = splits_noise(G.kind, sa.N, sa.nd, h->noise != 0) ? 1 : 0;
         sa.slice_opd_stride = slice_stride;
         sa.dyn[0] = dyn;
+        if (sa.split_noise && !dyn.st_E) sa.dyn[0].st_E = h->d_E;  // the noise pass reads E back
         if (slice_stride > 0) sa.dyn[0].opd = h->d_opd_sl;
         long sl = timed_begin(h, kind_name(G.kind) + std::to_string(sa.N), ls);
         cudaError_t err = launch_spot(G.kind, sa, ls, after_project && !h->timing);
@@ -820,7 +821,6 @@ void calib_free(CalibScratch &c) {
     cudaFree(c.d_wfs);
     cudaFree(c.d_inst);
     cudaFree(c.opd);
-    cudaFree(c.E);
     cudaFree(c.slopes);
     cudaFree(c.layers);
     cudaFree(c.work);
@@ -850,7 +850,6 @@ wfs_status calib_prepare(wfs_loop lp, int gs) {
     c.nv = base.n_valid;
     c.blocks_per_wfs = project_blocks(base);
     c.opd_stride = (size_t)c.nv * base.n * base.n;
-    c.det_stride = (size_t)c.nv * G.g.n_det * G.g.n_det;
     std::vector<WfsDesc> w(kMaxInstances, base);
     for (int i = 0; i < kMaxInstances; ++i) {
         w[i].inst = i;
@@ -877,7 +876,6 @@ wfs_status calib_prepare(wfs_loop lp, int gs) {
     if ((e = cudaMalloc(&c.d_wfs, sizeof(WfsDesc) * kMaxInstances)) != cudaSuccess) return bail(e, "calibration table");
     if ((e = cudaMalloc(&c.d_inst, sizeof(InstDesc) * in.size())) != cudaSuccess) return bail(e, "calibration table");
     if ((e = cudaMalloc(&c.opd, sizeof(float) * c.opd_stride * kMaxInstances)) != cudaSuccess ||
-        (e = cudaMalloc(&c.E, sizeof(float) * c.det_stride * kMaxInstances)) != cudaSuccess ||
         (e = cudaMalloc(&c.slopes, sizeof(float) * 2 * c.nv * kMaxInstances)) != cudaSuccess ||
         (e = cudaMalloc(&c.layers, sizeof(float) * SS * kMaxInstances)) != cudaSuccess ||
         (e = cudaMalloc(&c.work, sizeof(int) * 4)) != cudaSuccess)
@@ -1722,7 +1720,6 @@ wfs_status batch_fill(wfs_batch b, const float *const *screens, const double *t,
         d.slopes = slopes[i];
         d.t = t[i];
         d.noise = b->hs[i]->noise;
-        d.st_E = b->hs[i]->d_E;
         b->hs[i]->last_stream = nullptr;
     }
     bool aligned = true;
@@ -1730,9 +1727,15 @@ wfs_status batch_fill(wfs_batch b, const float *const *screens, const double *t,
     b->pa->stage_cap = (b->proj_stage > 0 && aligned) ? b->proj_stage : 0;
     for (size_t c = 0; c < b->classes.size(); ++c) {
         ShArgs &a = *b->sa[c];
+        const BatchClass &bc = b->classes[c];
         memcpy(a.dyn, b->pa->dyn, sizeof(InstDyn) * n);
-        a.grid_cap = b->classes[c].grid_cap;
-        a.cta_warps = b->classes[c].cta_warps;
+        bool noise = false;
+        for (int k = 0; k < bc.count; ++k) noise = noise || b->hs[b->wfs_host[bc.first + k].inst]->noise;
+        a.split_noise = splits_noise(bc.kind, a.N, a.nd, noise) ? 1 : 0;
+        if (a.split_noise)
+            for (int i = 0; i < n; ++i) a.dyn[i].st_E = b->hs[i]->d_E;
+        a.grid_cap = bc.grid_cap;
+        a.cta_warps = bc.cta_warps;
     }
     return WFS_OK;
 }
@@ -1977,7 +1980,6 @@ wfs_status wfs_batch_create(int n, const wfs_handle *hs, wfs_batch *out) {
         a->status = hs[0]->d_status;
         a->n_inst = n;
         a->work = b->d_work + 2 * b->sa.size();
-        a->split_noise = splits_noise(bc.kind, a->N, a->nd) ? 1 : 0;
         b->sa.push_back(a);
     }
     const char *g = getenv("GBWFS_BATCH_GRAPH");
@@ -2001,8 +2003,12 @@ wfs_status wfs_batch_measure(wfs_batch b, const float *const *screens, const dou
         if ((e = batch_launch_direct(b, s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
         return WFS_OK;
     }
-    // the projection node's kernel follows the screens' alignment: a change rebuilds the graph
-    if (b->exec && b->graph_stage != b->pa->stage_cap) batch_drop_graph(b);
+    // the projection node's kernel follows the screens' alignment, and a class has a noise node
+    // only while an instance of it has noise on: a change of either rebuilds the graph
+    bool same = b->graph_stage == b->pa->stage_cap;
+    for (size_t c = 0; c < b->classes.size() && c < b->noise_nodes.size(); ++c)
+        same = same && (b->classes[c].total <= 0 || (b->noise_nodes[c] != nullptr) == (b->sa[c]->split_noise != 0));
+    if (b->exec && !same) batch_drop_graph(b);
     if (!b->exec) {
         if ((e = batch_build_graph(b)) != cudaSuccess) {
             batch_drop_graph(b);
@@ -2060,7 +2066,6 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
             d.slopes = slopes_out[pos[i]];
             d.t = t_s[pos[i]];
             d.noise = b->hs[i]->noise;
-            d.st_E = b->hs[i]->d_E;
         }
     int count = 0, blocks = 0, box = 0, stage = 0;
     bool aligned = true;
@@ -2115,8 +2120,12 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
         sa.cta_warps = bc.cta_warps;
         sa.n_inst = n;
         sa.work = b->d_work + 2 * (b->classes.size() * (1 + (size_t)slot) + c);
-        sa.split_noise = splits_noise(bc.kind, sa.N, sa.nd) ? 1 : 0;
         memcpy(sa.dyn, pa.dyn, sizeof(InstDyn) * n);
+        bool noise = false;
+        for (int k = 0; k < cls_count[c]; ++k) noise = noise || b->hs[sl.h[cls_first[c] + k].inst]->noise;
+        sa.split_noise = splits_noise(bc.kind, sa.N, sa.nd, noise) ? 1 : 0;
+        if (sa.split_noise)
+            for (int i = 0; i < n; ++i) sa.dyn[i].st_E = b->hs[i]->d_E;
         if ((e = launch_spot(bc.kind, sa, (cudaStream_t)stream)) != cudaSuccess)
             return cuda_fail(nullptr, e, "batch subset spot launch");
         if (sa.split_noise && (e = launch_noise_cog(sa, (cudaStream_t)stream, false)) != cudaSuccess)
@@ -2424,7 +2433,6 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
                 dyn.dm = c.layers + i * SS;
                 dyn.opd = c.opd + i * c.opd_stride;
                 dyn.slopes = c.slopes + (size_t)i * n_slopes;
-                dyn.st_E = c.E + i * c.det_stride;
                 pa.dyn[i] = dyn;
             }
             sl = timed_begin(h, "project", s);
@@ -2443,16 +2451,10 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             sa.n_inst = ni;
             sa.work = c.work + 2;
             sa.project = 0;
-            sa.split_noise = splits_noise(c.kind, sa.N, sa.nd) ? 1 : 0;
-            memcpy(sa.dyn, pa.dyn, sizeof(InstDyn) * ni);
+            memcpy(sa.dyn, pa.dyn, sizeof(InstDyn) * ni);  // no noise: the spot kernel takes the centroids
             sl = timed_begin(h, kind_name(c.kind) + std::to_string(sa.N), s);
             e = launch_spot(c.kind, sa, s, !h->timing);
             timed_end(h, sl, s);
-            if (e == cudaSuccess && sa.split_noise) {
-                sl = timed_begin(h, "noise_cog", s);
-                e = launch_noise_cog(sa, s, !h->timing);
-                timed_end(h, sl, s);
-            }
             if (e != cudaSuccess) return cuda_fail(h, e, "calibration spot launch");
             sl = timed_begin(h, "push_pull_rows", s);
             e = launch_push_pull_rows(c.slopes, K, n_slopes, (float)(0.5 / amplitude),

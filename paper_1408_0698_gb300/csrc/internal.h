@@ -132,7 +132,8 @@ struct ShArgs {
     // s * slice_opd_stride floats after slice 0 (projected by k_project); 0 = one OPD
     long long slice_opd_stride;
     int split_noise;     // 32-point kernels: 1 = store the expected image (dyn.st_E, required)
-                         // and stop; launch_noise_cog completes the measurement
+                         // and stop; launch_noise_cog completes the measurement; 0 = no instance
+                         // has noise on: the centroid of the expected image in the spot kernel
     InstDyn dyn[kMaxInstances];
 };
 
@@ -274,9 +275,12 @@ cudaError_t launch_spot(int kind, const ShArgs &a, cudaStream_t s, bool after_pr
 // follows that spot kernel on s as a programmatic dependent launch.
 cudaError_t launch_noise_cog(const ShArgs &a, cudaStream_t s, bool after_spot);
 cudaError_t noise_cog_launch_shape(const ShArgs &a, LaunchShape *out);
-// Whether a spot kind stores expected images and leaves noise and centroid to k_noise_cog.
-// The 32-point kernels with a 16 x 16 detector leave the noise and the centroid to k_noise_cog.
-inline bool splits_noise(int kind, int N, int nd) { return (kind == kSpotN32 || is_tc(kind)) && N == 32 && nd == 16; }
+// Whether a spot launch stores expected images and leaves noise and centroid to k_noise_cog: the
+// 32-point kernels with a 16 x 16 detector, when an instance of the launch has noise on.  Without
+// noise the spot kernel takes the centroid itself (tail::finish).
+inline bool splits_noise(int kind, int N, int nd, bool noise) {
+    return noise && (kind == kSpotN32 || is_tc(kind)) && N == 32 && nd == 16;
+}
 // Swizzled BF16 (f16: FP16) operand tiles of the two constant matrices (F^T blocks, Ga blocks),
 // from FP64 tables laid out [q][m] (F) and [d][k] (Ga).
 void build_tc_tiles(int n, int N, const double *F_re64, const double *F_im64, const double *Ga_re64,

@@ -63,8 +63,7 @@ struct N32Layout {
     static constexpr int oGam = oFm + N * n;       // [m][dx]  Ga[dx][m]    (broadcast rows)
     static constexpr int oFft = oGam + N * n;      // lane-DFT twiddles and phases (tail::fill_fft_table)
     static constexpr int oG = oFft + tail::kFftTable;  // [d][nd]  G[d][i]
-    static constexpr int oRk = oG + n * nd;         // RN(1/k) for the Poisson inversion (floats)
-    static constexpr int table = oRk + kRecipTable / 2;
+    static constexpr int table = oG + n * nd;
     // per-warp scratch (float2 units)
     static constexpr int wX = 0;                   // [p][q]
     static constexpr int wTa = wX + n * n;         // Q: [nd][n]
@@ -96,8 +95,6 @@ __global__ void __launch_bounds__(256, 2) k_sh_n32(const __grid_constant__ ShArg
         Gam[k * n + d] = g;
     }
     for (int i = threadIdx.x; i < n * nd; i += blockDim.x) Gt[i] = a.G[i];
-    float *rk = reinterpret_cast<float *>(sm2 + Lay::oRk);
-    fill_recip_table(rk, threadIdx.x, blockDim.x);
     tail::fill_fft_table<n>(fft, threadIdx.x, blockDim.x);
     __syncthreads();
     wait_prior_grid();
@@ -116,9 +113,6 @@ __global__ void __launch_bounds__(256, 2) k_sh_n32(const __grid_constant__ ShArg
         if (a.work && lane == 0) ticket = atomicAdd(a.work, 1);
         const WfsDesc &W = a.wfs[find_wfs(a.wfs, a.n_wfs, g)];
         const InstDyn &D = a.dyn[W.inst];
-        const uint64_t seed = a.inst[W.inst].seed;
-        const uint32_t tlo = (uint32_t)__double_as_longlong(D.t);
-        const uint32_t thi = (uint32_t)((unsigned long long)__double_as_longlong(D.t) >> 32);
         const int v = g - W.subap_begin;
         __syncwarp();
         if (!guard(v >= 0 && v < W.n_valid, a.status)) {  // uniform over the warp
@@ -267,7 +261,7 @@ __global__ void __launch_bounds__(256, 2) k_sh_n32(const __grid_constant__ ShArg
             __syncwarp();
             tail::ngs_binned<nd>(Iw, lane, Bv);
         }
-        tail::finish<nd>(Bv, W, D, seed, v, lane, rk, a.split_noise != 0);
+        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
         g = a.work ? nwarps + __shfl_sync(0xffffffffu, ticket, 0) : g + nwarps;
     }
     if (a.work) {

@@ -137,8 +137,7 @@ struct TcLayout {
     static constexpr int tFft = tFk + (kMmaU ? 0 : n * N);  // lane-DFT twiddles and phases (tail::fill_fft_table)
     static constexpr int tG = tFft + (kLane ? tail::kFftTable : 0);  // [d][nd] G[d][i]
     static constexpr int tGa = tG + n * nd;        // [d][k] Ga (direct-sum stages only)
-    static constexpr int tRk = tGa + (kLane ? 0 : n * N);  // RN(1/k) for the Poisson inversion (floats)
-    static constexpr int tEnd = tRk + kRecipTable / 2;
+    static constexpr int tEnd = tGa + (kLane ? 0 : n * N);
     static constexpr int oWarp = (oTab + tEnd * 8 + 15) / 16 * 16;  // per-warp scratch (float2)
     static constexpr int even(int x) { return (x + 1) & ~1; }
     // 32-lane path: the NGS image rows (wI) alias the LGS scratch (wQ); X and Q hold column
@@ -191,7 +190,6 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     float2 *tab = reinterpret_cast<float2 *>(smem + Lay::oTab);
     float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft, *Gt = tab + Lay::tG;
     float2 *Gat = tab + Lay::tGa;
-    float *rk = reinterpret_cast<float *>(tab + Lay::tRk);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + 32 * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 20);  // next group (dynamic split)
@@ -225,7 +223,6 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         else
             for (int i = tid; i < n * N; i += kTcThreads) Gat[i] = a.Ga[i];
         for (int i = tid; i < n * nd; i += kTcThreads) Gt[i] = a.G[i];
-        fill_recip_table(rk, tid, kTcThreads);
     }
     if (wib == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -546,7 +543,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
                                         Kts, lane, Bv);
             } else
                 tail::ngs_binned<nd>(Iw, lane, Bv);
-            tail::finish<nd>(Bv, W, D, a.inst[W.inst].seed, v, lane, rk, a.split_noise != 0);
+            tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
         } else {
             float2 *wbase = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp;
             float *Bw;
@@ -603,7 +600,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
     uint8_t *sA1 = smem + Lay::oA + 16384 * wg, *sA2 = sA1;
     float2 *tab = reinterpret_cast<float2 *>(smem + Lay::oTab);
     float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft, *Gt = tab + Lay::tG;
-    float *rk = reinterpret_cast<float *>(tab + Lay::tRk);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + Lay::misc * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 20);  // next group (dynamic split)
@@ -627,7 +623,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         }
         tail::fill_fft_table<n>(fft, tid, kTcThreads);
         for (int i = tid; i < n * nd; i += kTcThreads) Gt[i] = a.G[i];
-        fill_recip_table(rk, tid, kTcThreads);
     }
     if (wib == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -925,7 +920,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
                                     lane, Bv);
         } else
             tail::ngs_binned<nd>(Iw, lane, Bv);
-        tail::finish<nd>(Bv, W, D, a.inst[W.inst].seed, v, lane, rk, a.split_noise != 0);
+        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy outlives the CTA
     fence_before_sync();

@@ -338,15 +338,40 @@ __device__ __forceinline__ void noise_centroid(const float (&ev)[nd / 2], const 
     }
 }
 
-// Photometry, noise and the centroid in one pass (the spot kernel completes the measurement);
-// with split, only the expected image is stored and the noise kernel completes it.
+// Photometry, then the centroid of the expected image in place (a measurement without noise); with
+// split, the expected image is stored and the noise kernel completes the measurement.  The sums of
+// the centroid run in noise_centroid's order.  Without noise the image would only travel to the
+// noise kernel and back: ELT frame, FP32, 125.5 us + 17.2 us for that pass -> 129.4 us in place, the frame 181.5 -> 172.7 us; the
+// 64-measurement chunk of a calibration 857 + 148 us -> 869 us.
 template <int nd>
-__device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc &W, const InstDyn &D,
-                                       uint64_t seed, int v, int lane, const float *rk, bool split) {
-    float ev[nd / 2];
+__device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc &W, const InstDyn &D, int v,
+                                       int lane, bool split) {
+    constexpr int nd2 = nd * nd, J = nd / 2;
+    const int ix = lane & 15, half = lane >> 4;
+    float ev[J];
     expected<nd>(Bv, W, v, lane, ev);
     store_expected<nd>(ev, W, D, v, lane);
-    if (!split) noise_centroid<nd>(ev, W, D, seed, v, lane, rk);
+    if (split) return;
+    const float cd = 0.5f * (float)(nd - 1);
+    float *st_C = D.st_C ? D.st_C + W.det_off + (size_t)v * nd2 : nullptr;
+    float sc = 0.0f, sx = 0.0f, sy = 0.0f;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const int iy = half * J + j;
+        if (st_C) st_C[iy * nd + ix] = ev[j];
+        sc += ev[j];
+        sx = fmaf((float)ix - cd, ev[j], sx);
+        sy = fmaf((float)iy - cd, ev[j], sy);
+    }
+    sc = warp_sum(sc);
+    sx = warp_sum(sx);
+    sy = warp_sum(sy);
+    if (lane == 0) {
+        const bool ok = sc > 0.0f;
+        float *sl = D.slopes + W.slope_off;
+        sl[2 * v] = ok ? sx / sc : 0.0f;
+        sl[2 * v + 1] = ok ? sy / sc : 0.0f;
+    }
 }
 
 // ---- any DFT size (N <= 32) and detector tile: the same stages as direct sums over the warp's
