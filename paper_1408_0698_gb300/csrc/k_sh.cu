@@ -486,12 +486,49 @@ cudaError_t launch_ktil(const KtilArgs &a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// The noise stage alone, for element-wise checks of the generator.
+// The noise stage alone.  A thread takes a pixel pair: one generator block and one Box-Muller
+// transform serve both pixels, and both inversion searches go through the packed warp search.
+// Issue-bound: 7.1 M pixels 102.4 -> 57.4 us (a thread per pixel formed its pair's block twice).
 // ---------------------------------------------------------------------------
-__global__ void k_noise(const float *E, int n, float ron, uint64_t seed, uint32_t wfs,
-                        uint32_t tlo, uint32_t thi, uint32_t pixel0, float *C) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) C[i] = noise_pixel(E[i], ron, seed, pixel0 + (uint32_t)i, wfs, tlo, thi);
+__global__ void __launch_bounds__(256) k_noise(const float *E, int n, float ron, uint64_t seed, uint32_t wfs,
+                                               uint32_t tlo, uint32_t thi, uint32_t pixel0, bool vec, float *C) {
+    __shared__ float4 rk2[kRecipTable / 2];
+    fill_recip_pairs(rk2, threadIdx.x, blockDim.x);
+    __syncthreads();
+    // pair j of the range: array elements i, i + 1 are its even and odd pixel (each if inside)
+    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long i = 2 * j - (long long)(pixel0 & 1u);
+    const bool in0 = i >= 0 && i < n, in1 = i + 1 < n;  // i >= -1
+    float2 e = make_float2(0.0f, 0.0f);
+    if (vec && in0 && in1) {
+        e = *reinterpret_cast<const float2 *>(E + i);
+    } else {
+        if (in0) e.x = E[i];
+        if (in1) e.y = E[i + 1];
+    }
+    const PairStream q = pair_stream(seed, pixel0 + (uint32_t)(in0 ? i : i + 1), wfs, tlo, thi);
+    const uint4 r = q.block(0);
+    float ze, zo;
+    box_muller_pair(r.x, r.y, ze, zo);
+    const float2 em = make_float2(inversion_mean(e.x), inversion_mean(e.y));
+    int k0, k1;
+    poisson_inversion_pair(em, make_float2(philox_unit(r.z), philox_unit(r.w)),
+                           make_float2(expf(-em.x), expf(-em.y)), rk2, k0, k1);
+    for (int s = 0; s < 2; ++s) {  // one PTRS call site
+        const float es = s ? e.y : e.x;
+        if (es >= 16.0f) {
+            const int k = poisson_ptrs(es, q, s);
+            if (s) k1 = k;
+            else k0 = k;
+        }
+    }
+    const float2 c = make_float2((float)k0 + ron * ze, (float)k1 + ron * zo);
+    if (vec && in0 && in1) {
+        *reinterpret_cast<float2 *>(C + i) = c;
+    } else {
+        if (in0) C[i] = c.x;
+        if (in1) C[i + 1] = c.y;
+    }
 }
 
 cudaError_t launch_noise(const float *E, int n, float ron, uint64_t seed, uint32_t wfs, double t,
@@ -499,8 +536,11 @@ cudaError_t launch_noise(const float *E, int n, float ron, uint64_t seed, uint32
     if (n <= 0) return cudaSuccess;
     unsigned long long tb;
     memcpy(&tb, &t, sizeof tb);
-    k_noise<<<(n + 255) / 256, 256, 0, s>>>(E, n, ron, seed, wfs, (uint32_t)tb,
-                                            (uint32_t)(tb >> 32), pixel0, C);
+    // 8-byte accesses where the pairs start on 8-byte boundaries of both arrays
+    const bool vec = (pixel0 & 1u) == 0 && ((reinterpret_cast<uintptr_t>(E) | reinterpret_cast<uintptr_t>(C)) & 7) == 0;
+    const long long pairs = ((long long)(pixel0 & 1u) + n + 1) / 2;
+    k_noise<<<(unsigned)((pairs + 255) / 256), 256, 0, s>>>(E, n, ron, seed, wfs, (uint32_t)tb, (uint32_t)(tb >> 32),
+                                                            pixel0, vec, C);
     return cudaGetLastError();
 }
 

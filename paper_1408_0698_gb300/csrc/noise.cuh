@@ -19,7 +19,7 @@
 // random variables", 1993).  The integer decisions are taken in FP32 with
 // explicitly rounded operations (no contraction), so the operation order is
 // fixed.  For E < 16 the search stops before k = 43 even at the largest
-// uniform, so RN(1/k) fits a 64-entry table.
+// uniform, so RN(1/k) fits a 64-entry table (poisson_inversion_pair).
 //
 // Everything here works on values: no generator object lives in memory, so a
 // warp can run the generator blocks of several pixels side by side.
@@ -28,7 +28,7 @@
 
 namespace gbwfs {
 
-constexpr int kRecipTable = 64;  // RN(1/k), k < 64 (entry 0 unused)
+constexpr int kRecipTable = 64;  // RN(1/k), k <= 64
 
 // Philox4x32-10 of counter (x0, x1, x2, x3) under key (k0, k1).
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
@@ -95,31 +95,9 @@ __device__ __forceinline__ float log_factorial_f32(float k) {
 }
 
 // Inversion for 0 < E < 16 with the first Poisson uniform u and p0 = exp(-E): the smallest k
-// with u <= F_k, F_k = F_{k-1} + p_k, stopping early where F stops growing.  With TAB, rk[k]
-// holds RN(1/k) for k < kRecipTable, and the loop takes two steps a trip (both steps' table
-// entries loaded together, the second step's result dropped when the first stops): the search
-// ends before k = 43 for every E < 16 (and only finite 0 < E < 16 reach it), so no read passes
-// entry 43.  Otherwise 1/k is rounded on the spot.  Both forms take the same operations in the
-// same order.
-template <bool TAB>
-__device__ __forceinline__ int poisson_inversion(float E, float u, float p0, const float *rk) {
+// with u <= F_k, F_k = F_{k-1} + p_k, stopping early where F stops growing.
+__device__ __forceinline__ int poisson_inversion(float E, float u, float p0) {
     float p = p0, F = p0;
-    if (TAB) {
-        if (!(u > F)) return 0;
-        for (int k = 1;; k += 2) {
-            const float r1 = rk[k], r2 = rk[k + 1];
-            const float p1 = __fmul_rn(__fmul_rn(p, E), r1);
-            const float F1 = __fadd_rn(F, p1);
-            const bool s1 = F1 == F || !(u > F1);
-            const float p2 = __fmul_rn(__fmul_rn(p1, E), r2);
-            const float F2 = __fadd_rn(F1, p2);
-            const bool s2 = F2 == F1 || !(u > F2);
-            if (s1) return k;
-            if (s2) return k + 1;
-            p = p2;
-            F = F2;
-        }
-    }
     int k = 0;
     while (u > F) {
         k = k + 1;
@@ -130,6 +108,45 @@ __device__ __forceinline__ int poisson_inversion(float E, float u, float p0, con
         F = Fn;
     }
     return k;
+}
+
+// The same searches for two pixels of every lane of a converged warp (E = 0 for a pixel without a
+// draw: count 0), the pair in packed FP32x2 (each half rounded as the scalar operation).  F never
+// decreases, so k is the number of indices j >= 0 with u > F_j and no lane needs to stop: the sign
+// of F_j - u is added up and the warp leaves after the first group of four indices that no lane
+// counts in.  A lane that stops because F no longer grows still has u > F at the end (p only
+// shrinks from there on) and is redone by the scalar search; so is any lane past the table.  rk2:
+// fill_recip_pairs, in shared memory.
+// Issue-bound: 7.5 instructions per index of two pixels, against 8 per index of one for a scalar
+// loop of two indices a trip; leaving after pairs of indices instead of groups of four was no faster.
+__device__ __forceinline__ void poisson_inversion_pair(float2 E, float2 u, float2 p0, const float4 *rk2, int &k0,
+                                                       int &k1) {
+    const float2 nu = make_float2(-u.x, -u.y);
+    float2 p = p0, F = p0, d = __fadd2_rn(F, nu);
+    int c0 = -(__float_as_int(d.x) >> 31), c1 = -(__float_as_int(d.y) >> 31);
+    for (int k = 0; k < kRecipTable / 2; k += 2) {  // indices 2k + 1 .. 2k + 4
+        if (!__any_sync(0xffffffffu, fminf(d.x, d.y) < 0.0f)) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 r = rk2[k + h];
+            p = __fmul2_rn(__fmul2_rn(p, E), make_float2(r.x, r.y));
+            F = __fadd2_rn(F, p);
+            d = __fadd2_rn(F, nu);
+            c0 -= __float_as_int(d.x) >> 31;
+            c1 -= __float_as_int(d.y) >> 31;
+            p = __fmul2_rn(__fmul2_rn(p, E), make_float2(r.z, r.w));
+            F = __fadd2_rn(F, p);
+            d = __fadd2_rn(F, nu);
+            c0 -= __float_as_int(d.x) >> 31;
+            c1 -= __float_as_int(d.y) >> 31;
+        }
+    }
+    if (fminf(d.x, d.y) < 0.0f) {  // about one draw in 2^23
+        if (d.x < 0.0f) c0 = poisson_inversion(E.x, u.x, p0.x);
+        if (d.y < 0.0f) c1 = poisson_inversion(E.y, u.y, p0.y);
+    }
+    k0 = c0;
+    k1 = c1;
 }
 
 // PTRS for E >= 16: draws word 2 + parity of block 0, then blocks 1 + parity, 3 + parity,
@@ -174,11 +191,9 @@ __device__ __forceinline__ int poisson_ptrs(float E, const PairStream &q, int pa
 
 // Poisson count of a pixel of the given parity whose block 0 gave the inversion uniform u
 // (word 2 + parity).
-template <bool TAB>
-__device__ __forceinline__ int poisson_count(float E, float u, float p0, const PairStream &q, int parity,
-                                             const float *rk) {
+__device__ __forceinline__ int poisson_count(float E, float u, float p0, const PairStream &q, int parity) {
     if (!(E > 0.0f)) return 0;
-    if (E < 16.0f) return poisson_inversion<TAB>(E, u, p0, rk);
+    if (E < 16.0f) return poisson_inversion(E, u, p0);
     return poisson_ptrs(E, q, parity);
 }
 
@@ -191,13 +206,20 @@ __device__ __forceinline__ float noise_pixel(float E, float read_noise, uint64_t
     const int parity = (int)(pixel & 1u);
     float ze, zo;
     box_muller_pair(r.x, r.y, ze, zo);
-    const int k = poisson_count<false>(E, philox_unit(parity ? r.w : r.z), expf(-E), q, parity, nullptr);
+    const int k = poisson_count(E, philox_unit(parity ? r.w : r.z), expf(-E), q, parity);
     return (float)k + read_noise * (parity ? zo : ze);
 }
 
-// Fills rk[0 .. kRecipTable) with RN(1/k) (entry 0 = 1); call from every thread of the block.
-__device__ __forceinline__ void fill_recip_table(float *rk, int tid, int nthreads) {
-    for (int i = tid; i < kRecipTable; i += nthreads) rk[i] = __frcp_rn((float)(i > 0 ? i : 1));
+// The mean of an inversion search: E where the search applies, 0 (no draw) elsewhere.
+__device__ __forceinline__ float inversion_mean(float E) { return E > 0.0f && E < 16.0f ? E : 0.0f; }
+
+// Fills rk2[i], i < kRecipTable / 2, with RN(1/k) twice for k = 2i + 1 and twice for 2i + 2; call
+// from every thread of the block.
+__device__ __forceinline__ void fill_recip_pairs(float4 *rk2, int tid, int nthreads) {
+    for (int i = tid; i < kRecipTable / 2; i += nthreads) {
+        const float a = __frcp_rn((float)(2 * i + 1)), b = __frcp_rn((float)(2 * i + 2));
+        rk2[i] = make_float4(a, a, b, b);
+    }
 }
 
 }  // namespace gbwfs

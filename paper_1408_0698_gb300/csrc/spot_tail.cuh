@@ -250,82 +250,94 @@ __device__ __forceinline__ void store_expected(const float (&ev)[nd / 2], const 
     for (int j = 0; j < J; ++j) st_E[(half * J + j) * nd + ix] = ev[j];
 }
 
-// Noise and the centroid of subaperture v of WFS W from its expected image ev (the layout of
-// expected()); lane 0 writes the slopes.  rk: RN(1/k) table (fill_recip_table) in shared
-// memory.  One generator block per pixel pair; each exchange between the lane pair is followed
-// by both pixels' inversion searches, and the rare pixels with E >= 16 go last through one PTRS
-// call site.
+// The detector row of a lane's slot j in the noise pass.  Without noise, the layout of expected().
+// With noise, slots m and m + nd/4 (searched together) hold neighbouring rows, and the two
+// half-warps take rows mirrored about the centre, so that the rows a warp searches together are
+// about as bright: its search lasts as long as its brightest pixel's.
+template <int nd>
+__device__ __forceinline__ int noise_row(int j, int half, bool noise) {
+    constexpr int J = nd / 2;
+    if (!noise) return half * J + j;
+    const int r = 2 * (j & (J / 2 - 1)) + j / (J / 2);
+    return half ? nd - 1 - r : r;
+}
+
+// Noise and the centroid of subaperture v of WFS W from its expected image ev (row noise_row of
+// slot j); lane 0 writes the slopes.  rk2: fill_recip_pairs.  One generator block per pixel pair;
+// each exchange between the lane pair is followed by both pixels' inversion searches, and the rare
+// pixels with E >= 16 go last through one PTRS call site.  Call from the whole warp.
 template <int nd>
 __device__ __forceinline__ void noise_centroid(const float (&ev)[nd / 2], const WfsDesc &W, const InstDyn &D,
-                                               uint64_t seed, int v, int lane, const float *rk) {
+                                               uint64_t seed, int v, int lane, const float4 *rk2) {
     constexpr int nd2 = nd * nd, J = nd / 2;
     static_assert(nd == 16, "pixel pairs are the lane pairs (ix, ix + 1) of a 16-lane row");
     const int ix = lane & 15, half = lane >> 4;
+    const bool noise = D.noise != 0;
     const float cd = 0.5f * (float)(nd - 1);
     const uint32_t tlo = (uint32_t)__double_as_longlong(D.t);
     const uint32_t thi = (uint32_t)((unsigned long long)__double_as_longlong(D.t) >> 32);
-    float *st_C = D.st_C ? D.st_C + W.det_off : nullptr;
+    float *st_C = D.st_C ? D.st_C + W.det_off + (size_t)v * nd2 : nullptr;
     float sc = 0.0f, sx = 0.0f, sy = 0.0f;
-    if (ix < nd) {
-        float cv[J];
-        if (D.noise) {
-            // Pixel pairs (2m, 2m + 1) are the lanes (ix, ix + 1) of one row: the even lane
-            // forms the pair blocks of its first J/2 rows, the odd lane those of its last J/2,
-            // and each hands its partner that pixel's deviate and uniform; rows m and
-            // m + J/2 are then sampled together.
-            const uint32_t pix0 = (uint32_t)(v * nd2 + half * J * nd + ix);
-            const int par = ix & 1;
-            uint32_t big = 0;
-            float z[J];
+    float cv[J];
+    if (noise) {
+        // Pixel pairs (2m, 2m + 1) are the lanes (ix, ix + 1) of one row: the even lane forms the
+        // pair blocks of its first J/2 slots, the odd lane those of its last J/2, and each hands
+        // its partner that pixel's deviate and uniform; slots m and m + J/2 are then sampled
+        // together.
+        const uint32_t pix0 = (uint32_t)(v * nd2 + ix);
+        const int par = ix & 1;
+        uint32_t big = 0;
+        float z[J];
 #pragma unroll
-            for (int m = 0; m < J / 2; ++m) {
-                const uint32_t pix = pix0 + (uint32_t)((par * (J / 2) + m) * nd);
-                const uint4 r = pair_stream(seed, pix, (uint32_t)W.gs_index, tlo, thi).block(0);
-                float ze, zd;
-                box_muller_pair(r.x, r.y, ze, zd);
-                const float zr = __shfl_xor_sync(0xffffffffu, par ? ze : zd, 1);
-                const float ur = __shfl_xor_sync(0xffffffffu, philox_unit(par ? r.z : r.w), 1);
-                const float zo = par ? zd : ze, uo = philox_unit(par ? r.w : r.z);
-                z[m] = par ? zr : zo;
-                z[m + J / 2] = par ? zo : zr;
-                const float ua = par ? ur : uo, ub = par ? uo : ur;
-                const float ea = ev[m], eb = ev[m + J / 2];
-                int ka = 0, kb = 0;
-                if (ea >= 16.0f) big |= 1u << m;
-                else if (ea > 0.0f) ka = poisson_inversion<true>(ea, ua, expf(-ea), rk);
-                if (eb >= 16.0f) big |= 1u << (m + J / 2);
-                else if (eb > 0.0f) kb = poisson_inversion<true>(eb, ub, expf(-eb), rk);
-                cv[m] = (float)ka + W.read_noise * z[m];
-                cv[m + J / 2] = (float)kb + W.read_noise * z[m + J / 2];
-            }
-            while (big) {  // PTRS: one call site, rare
-                const int j = __ffs(big) - 1;
-                big &= big - 1;
-                float e = 0.0f, zj = 0.0f;
-#pragma unroll
-                for (int jj = 0; jj < J; ++jj)
-                    if (jj == j) {
-                        e = ev[jj];
-                        zj = z[jj];
-                    }
-                const PairStream q = pair_stream(seed, pix0 + (uint32_t)(j * nd), (uint32_t)W.gs_index, tlo, thi);
-                const float c = (float)poisson_ptrs(e, q, par) + W.read_noise * zj;
-#pragma unroll
-                for (int jj = 0; jj < J; ++jj)
-                    if (jj == j) cv[jj] = c;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < J; ++j) cv[j] = ev[j];
+        for (int m = 0; m < J / 2; ++m) {
+            const uint32_t pix = pix0 + (uint32_t)(nd * (par ? noise_row<nd>(m + J / 2, half, true)
+                                                             : noise_row<nd>(m, half, true)));
+            const uint4 r = pair_stream(seed, pix, (uint32_t)W.gs_index, tlo, thi).block(0);
+            float ze, zd;
+            box_muller_pair(r.x, r.y, ze, zd);
+            const float zr = __shfl_xor_sync(0xffffffffu, par ? ze : zd, 1);
+            const float ur = __shfl_xor_sync(0xffffffffu, philox_unit(par ? r.z : r.w), 1);
+            const float zo = par ? zd : ze, uo = philox_unit(par ? r.w : r.z);
+            z[m] = par ? zr : zo;
+            z[m + J / 2] = par ? zo : zr;
+            const float ea = ev[m], eb = ev[m + J / 2];
+            if (ea >= 16.0f) big |= 1u << m;
+            if (eb >= 16.0f) big |= 1u << (m + J / 2);
+            const float2 e = make_float2(inversion_mean(ea), inversion_mean(eb));
+            int ka, kb;
+            poisson_inversion_pair(e, make_float2(par ? ur : uo, par ? uo : ur),
+                                   make_float2(expf(-e.x), expf(-e.y)), rk2, ka, kb);
+            cv[m] = (float)ka + W.read_noise * z[m];
+            cv[m + J / 2] = (float)kb + W.read_noise * z[m + J / 2];
         }
+        while (big) {  // PTRS: one call site, rare
+            const int j = __ffs(big) - 1;
+            big &= big - 1;
+            float e = 0.0f, zj = 0.0f;
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const int iy = half * J + j, o = iy * nd + ix;
-            if (st_C) st_C[(size_t)v * nd2 + o] = cv[j];
-            sc += cv[j];
-            sx = fmaf((float)ix - cd, cv[j], sx);
-            sy = fmaf((float)iy - cd, cv[j], sy);
+            for (int jj = 0; jj < J; ++jj)
+                if (jj == j) {
+                    e = ev[jj];
+                    zj = z[jj];
+                }
+            const PairStream q = pair_stream(seed, pix0 + (uint32_t)(nd * noise_row<nd>(j, half, true)),
+                                             (uint32_t)W.gs_index, tlo, thi);
+            const float c = (float)poisson_ptrs(e, q, par) + W.read_noise * zj;
+#pragma unroll
+            for (int jj = 0; jj < J; ++jj)
+                if (jj == j) cv[jj] = c;
         }
+    } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) cv[j] = ev[j];
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const int iy = noise_row<nd>(j, half, noise), o = iy * nd + ix;
+        if (st_C) st_C[o] = cv[j];
+        sc += cv[j];
+        sx = fmaf((float)ix - cd, cv[j], sx);
+        sy = fmaf((float)iy - cd, cv[j], sy);
     }
     sc = warp_sum(sc);
     sx = warp_sum(sx);
@@ -341,8 +353,8 @@ __device__ __forceinline__ void noise_centroid(const float (&ev)[nd / 2], const 
 // Photometry, then the centroid of the expected image in place (a measurement without noise); with
 // split, the expected image is stored and the noise kernel completes the measurement.  The sums of
 // the centroid run in noise_centroid's order.  Without noise the image would only travel to the
-// noise kernel and back: ELT frame, FP32, 125.5 us + 17.2 us for that pass -> 129.4 us in place, the frame 181.5 -> 172.7 us; the
-// 64-measurement chunk of a calibration 857 + 148 us -> 869 us.
+// noise kernel and back: ELT frame, FP32, 125.5 us + 17.2 us for that pass -> 129.4 us in place
+// (the frame 181.5 -> 172.7 us); a calibration's chunk of 64 measurements 857 + 148 us -> 869 us.
 template <int nd>
 __device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc &W, const InstDyn &D, int v,
                                        int lane, bool split) {

@@ -1,4 +1,5 @@
-"""The choice between the noise pass and the centroid in the spot kernel (32-point geometries; GPU)."""
+"""The noise stage's pair kernel at the edges of its range, and the choice between the noise pass
+and the centroid in the spot kernel (32-point geometries; GPU)."""
 import dataclasses
 
 import numpy as np
@@ -8,6 +9,34 @@ import torch
 from paper_1408_0698_gb300 import inputs, native
 
 pytestmark = pytest.mark.gpu
+
+
+def _noise(e, pixel0, offset=0, ron=2.5):
+    buf_e = torch.zeros(e.numel() + offset, device="cuda")
+    buf_c = torch.full((e.numel() + offset,), float("nan"), device="cuda")
+    buf_e[offset:] = e
+    native.wfs_noise_apply(buf_e[offset:].data_ptr(), e.numel(), ron, 77, 3, 0.125, pixel0,
+                           buf_c[offset:].data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.isnan(buf_c[:offset]).all()
+    return buf_c[offset:].cpu().numpy()
+
+
+@pytest.mark.parametrize("first,count,offset", [(0, 1, 0), (1, 1, 0), (1, 2, 1), (0, 3, 1), (5, 62, 0), (7, 511, 3),
+                                                (64, 513, 1), (0xFFFFFFFD - 1000, 1000, 0)])
+def test_noise_range_is_a_slice_of_the_whole(first, count, offset):
+    # a pixel's noise depends on its index alone, whatever range, alignment or neighbour it is drawn with
+    base = max(0, first - 3) & ~1
+    e = torch.as_tensor(inputs.random_expected_image(first - base + count + 5, 11)).cuda()
+    whole = _noise(e, base)
+    part = _noise(e[first - base: first - base + count], first, offset)
+    np.testing.assert_array_equal(part, whole[first - base: first - base + count])
+
+
+def test_noise_of_means_without_a_draw_and_large_means():
+    e = torch.tensor([0.0, -1.0, float("nan"), 15.999999, 16.0, 1e-30, 400.0, 3e-8], device="cuda")
+    c = _noise(e, 0, ron=0.0)
+    assert np.all(c[[0, 1, 2, 5]] == 0.0) and np.all(c >= 0.0) and np.all(c == np.rint(c)) and c[6] > 200
 
 
 def _elt_small(n, lgs, precision):
