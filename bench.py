@@ -84,7 +84,10 @@ def spot_flops(n, N, nd, lgs, kernel=""):
       4 nd^2 n; photometry 2 nd^2 (the centroid, 4 nd^2, runs in the separate noise pass);
       other sizes (direct sums): M (2n-1) n (8N+6); P = M G 8 (2n-1) nd n; B 4 nd^2 (2n-1);
       photometry and centroid 6 nd^2.
-    NGS: binning N^2, photometry and centroid 6 nd^2.  Without a kernel name, every stage dense."""
+    NGS: binning N^2, photometry and centroid 6 nd^2.  Without a kernel name, every stage dense.
+    The warp-per-subaperture FP32 kernel ("spot_row") is counted by row_flops."""
+    if kernel.startswith("spot_row"):
+        return row_flops(n, N, nd, lgs)
     fm = dft_forms(kernel, N)
     f = (4 * N * n * n + 2 * N * n if fm["U"] == "r2" else 8 * N * n * n)
     f += (2 * N * N * n + 4 * N * N if fm["Y"] == "r4" else 8 * N * N * n) + 3 * N * N
@@ -98,6 +101,23 @@ def spot_flops(n, N, nd, lgs, kernel=""):
     else:
         f += N * N + 6 * nd * nd
     return f
+
+
+def row_flops(n, N, nd, lgs):
+    """FP32 flops (FMA = 2) of one subaperture in the warp-per-subaperture FP32 kernel, whose centred
+    DFTs are folded about their centres (h = ceil(n/2) mirrored inputs, half of the outputs computed,
+    each giving its mirror by one more complex add): U 4Nhn + 4Nn; the fold of U 4Nh; Y per row and
+    column pair 8h + 4 adds, two |.|^2 of 3; LGS: T 2 adds and 4n per column pair (half of the 4n
+    where N is a multiple of 4, after 6 more adds per two pairs), its fold 4Nn, A 8 per (dy, dx) and
+    row pair and 4 adds, M 12 for each of +-dy and 4 adds, Q 8 per (dy, dx) and row pair and 4 adds,
+    B 4 per (dx, iy) and column pair and 2 adds; NGS: binning N^2.  Photometry and centroid 6 nd^2."""
+    h, hN, hd = (n + 1) // 2, (N + 1) // 2, (nd + 1) // 2
+    f = 4 * N * h * n + 4 * N * n + 4 * N * h + N * hN * (8 * h + 4 + 6)
+    if not lgs:
+        return f + N * N + 6 * nd * nd
+    f += N * (hN // 2) * (4 + 6 + 4 * n) if N % 4 == 0 else N * hN * (2 + 4 * n)
+    f += 4 * N * n + n * n * (8 * hN + 4 + 24 + 4) + hd * n * (8 * n + 4) + nd * hd * (4 * n + 2)
+    return f + 6 * nd * nd
 
 
 def dft_useful_flops(n, N):
@@ -137,7 +157,7 @@ def source_sha(names):
 
 
 KERNEL_SOURCES = {"spot": ["k_sh.cu", "noise.cuh", "proj_math.cuh", "internal.h"],
-                  "spot_n32": ["k_sh_n32.cu", "spot_tail.cuh", "noise.cuh", "internal.h"],
+                  "spot_row": ["k_sh_row.cu", "self_project.cuh", "proj_math.cuh", "spot_tail.cuh", "noise.cuh", "internal.h"],
                   "spot_tc": ["k_sh_tc.cu", "spot_tail.cuh", "noise.cuh", "internal.h", "tcgen05.cuh"],
                   "spot_tc64": ["k_sh_tc64.cu", "noise.cuh", "proj_math.cuh", "internal.h", "tcgen05.cuh"],
                   "noise_cog": ["k_noise_cog.cu", "spot_tail.cuh", "noise.cuh", "internal.h"],
@@ -737,7 +757,7 @@ def spot_roofline(name, timing, cfg, w, pk, kind):
     ach = cuda / avg_s / 1e12
     roof = {"kernel": name, "bound": "alu", "achieved": ach, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": ach / FP32_PEAK_TFLOPS,
-            "traffic": ncu_traffic("spot_n32" if name.startswith("spot_n32") else
+            "traffic": ncu_traffic("spot_row" if name.startswith("spot_row") else
                                    "spot_tc" if name.startswith("spot_tc") else "spot"),
             "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz",
             "flops_per_launch": cuda, "flops_note": "CUDA-core flops only (the MMA stages excluded)",

@@ -84,7 +84,7 @@ struct SpotGroup {
 int spot_kind(const wfs_geometry &g) {
     if (g.precision == WFS_PREC_BF16X3) return kSpotTc;
     if (g.precision == WFS_PREC_FP16S) return kSpotTcF16;
-    return sh_n32_supported(g.n_pix_sub, g.n_fft, g.n_det) ? kSpotN32 : kSpotGeneric;
+    return sh_row_supported(g.n_pix_sub, g.n_fft) ? kSpotRow : kSpotGeneric;
 }
 
 struct GsDev {
@@ -526,7 +526,7 @@ void fill_geom_args(ShArgs &sa, const GeomDev &G) {
 const char *kind_name(int kind) {
     return kind == kSpotTc      ? "spot_tc_bf16x3_N"
            : kind == kSpotTcF16 ? "spot_tc_fp16s_N"
-           : kind == kSpotN32   ? "spot_n32_fp32_N"
+           : kind == kSpotRow   ? "spot_row_fp32_N"
                                 : "spot_fp32_N";
 }
 
@@ -650,9 +650,11 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         for (int q = 0; q < G.count; ++q) needs_uplink |= h->wfs_host[G.first + q].uplink != nullptr;
         if (needs_uplink && (e = cudaStreamWaitEvent(ss, h->ev_uplink, 0)) != cudaSuccess)
             return cuda_fail(h, e, "uplink wait");
-        // a generic-kernel group (a few NGS subapertures) projects inside its spot kernel: one
-        // launch that starts with the call and owns its SMs only while it runs
-        const bool fused = G.kind == kSpotGeneric || G.per_slice || (is_tc(G.kind) && h->geoms[G.geom].g.n_fft == 64);
+        // a small FP32 group (a few NGS subapertures) or a 64-point one projects inside its spot
+        // kernel: one launch that starts with the call and owns its SMs only while it runs
+        const wfs_geometry &geo = h->geoms[G.geom].g;
+        const bool fused = G.kind == kSpotGeneric || G.per_slice || (is_tc(G.kind) && geo.n_fft == 64) ||
+                           (G.kind == kSpotRow && !(geo.n_fft == 32 && geo.n_det == 16));
         if (!fused && (e = project(G, ss)) != cudaSuccess) return cuda_fail(h, e, "projection launch");
         if ((e = launch_group(G, ss, !fused && G.proj_count > 0, fused ? 1 : 0)) != cudaSuccess)
             return cuda_fail(h, e, "spot launch");
@@ -2150,7 +2152,7 @@ wfs_status wfs_batch_tune(wfs_batch b, const float *const *screens, const double
         BatchClass &bc = b->classes[c];
         if (bc.total <= 0) continue;
         std::vector<std::pair<int, int>> cand;  // (grid cap, warps per CTA)
-        if (bc.kind == kSpotN32) {
+        if (bc.kind == kSpotRow) {
             for (int w : {4, 8})
                 for (int m : {2, 4, 8, 16}) cand.push_back({152 * m * (8 / w), w});
         } else if (is_tc(bc.kind) && bc.geom->g.n_fft == 64) {
@@ -2559,11 +2561,11 @@ wfs_status wfs_set_lgs_model(wfs_handle h, int per_slice) {
             G.base_kind = G.kind;
             G.base_grid_cap = G.grid_cap;
             G.base_cta_warps = G.cta_warps;
-            // the per-slice variant of the geometry's 32-point kernel (tensor-core or FP32) where
-            // it has one, else the self-projecting generic kernel
+            // the per-slice variant of the geometry's tensor-core kernel where it has one, else the
+            // FP32 kernel with a warp per subaperture, else the self-projecting generic kernel
             const wfs_geometry &geo = h->geoms[G.geom].g;
             if (!is_tc(G.kind) || !sh_tc_slices_supported(geo.n_pix_sub, geo.n_fft, geo.n_det))
-                G.kind = sh_n32_supported(geo.n_pix_sub, geo.n_fft, geo.n_det) ? kSpotN32 : kSpotGeneric;
+                G.kind = sh_row_supported(geo.n_pix_sub, geo.n_fft) ? kSpotRow : kSpotGeneric;
             G.grid_cap = G.cta_warps = 0;
         } else {
             G.kind = G.base_kind;
@@ -2578,7 +2580,7 @@ wfs_status wfs_set_lgs_model(wfs_handle h, int per_slice) {
             d.slices = per_slice ? h->d_slices + d.gs_index : nullptr;
             d.ktil = per_slice ? gd.d_ktil_g : gd.d_ktil;
         }
-        G.sl_projected = per_slice && (is_tc(G.kind) || G.kind == kSpotN32);
+        G.sl_projected = per_slice && (is_tc(G.kind) || G.kind == kSpotRow);
     }
     if (build_slice_projection(h) != WFS_OK) return WFS_ECUDA;
     if ((e = cudaMemcpy(h->d_wfs, h->wfs_host.data(), sizeof(WfsDesc) * h->wfs_host.size(), cudaMemcpyHostToDevice)) !=

@@ -128,8 +128,8 @@ struct ShArgs {
                          // itself (no separate projection launch; written to dyn.opd too) on a
                          // side stream, with the shared-memory reservation that keeps projection
                          // CTAs off its SMs; 2 = the same without the reservation
-    // 32-point kernels, LGS per-slice model: slice s of a subaperture's OPD sits
-    // s * slice_opd_stride floats after slice 0 (projected by k_project); 0 = one OPD
+    // LGS per-slice model on kernels that read projected slices: slice s of a subaperture's OPD
+    // sits s * slice_opd_stride floats after slice 0; 0 = one OPD
     long long slice_opd_stride;
     int split_noise;     // 32-point kernels: 1 = store the expected image (dyn.st_E, required)
                          // and stop; launch_noise_cog completes the measurement; 0 = no instance
@@ -256,11 +256,11 @@ int segment_max_count(int n);
 cudaError_t launch_ktil(const KtilArgs &a, cudaStream_t s);
 cudaError_t launch_noise(const float *E, int n, float ron, uint64_t seed, uint32_t wfs, double t,
                          uint32_t pixel0, float *C, cudaStream_t s);
-// Spot kernels: kind 0 = generic FP32 (any geometry), 1 = FP32 specialised for N = 32,
-// 2 = tensor core (BF16 x3) for N = 32, 3 = tensor core (scaled FP16 x3) for N = 32.
-enum SpotKind { kSpotGeneric = 0, kSpotN32 = 1, kSpotTc = 2, kSpotTcF16 = 3 };
+// Spot kernels: kind 0 = generic FP32 (any geometry), 1 = FP32 with a warp per subaperture
+// (N <= 32, 3 <= n <= 16), 2 = tensor core (BF16 x3), 3 = tensor core (scaled FP16 x3).
+enum SpotKind { kSpotGeneric = 0, kSpotRow = 1, kSpotTc = 2, kSpotTcF16 = 3 };
 inline bool is_tc(int kind) { return kind == kSpotTc || kind == kSpotTcF16; }
-bool sh_n32_supported(int n, int N, int nd);
+bool sh_row_supported(int n, int N);
 bool sh_tc_supported(int n, int N, int nd);
 bool sh_tc_slices_supported(int n, int N, int nd);
 // The 64-point tensor-core kernel (32 x 32 pupil pixels, 32 x 32 detector; NGS only).
@@ -276,10 +276,11 @@ cudaError_t launch_spot(int kind, const ShArgs &a, cudaStream_t s, bool after_pr
 cudaError_t launch_noise_cog(const ShArgs &a, cudaStream_t s, bool after_spot);
 cudaError_t noise_cog_launch_shape(const ShArgs &a, LaunchShape *out);
 // Whether a spot launch stores expected images and leaves noise and centroid to k_noise_cog: the
-// 32-point kernels with a 16 x 16 detector, when an instance of the launch has noise on.  Without
-// noise the spot kernel takes the centroid itself (tail::finish).
+// 32-point tensor-core kernels with a 16 x 16 detector, when an instance of the launch has noise on
+// (their warps run in lock step and would wait for each other's Poisson searches).  Without noise
+// they take the centroid themselves (tail::finish).
 inline bool splits_noise(int kind, int N, int nd, bool noise) {
-    return noise && (kind == kSpotN32 || is_tc(kind)) && N == 32 && nd == 16;
+    return noise && is_tc(kind) && N == 32 && nd == 16;
 }
 // Swizzled BF16 (f16: FP16) operand tiles of the two constant matrices (F^T blocks, Ga blocks),
 // from FP64 tables laid out [q][m] (F) and [d][k] (Ga).

@@ -23,6 +23,7 @@
 #include "internal.h"
 #include "noise.cuh"
 #include "proj_math.cuh"
+#include "self_project.cuh"
 
 namespace gbwfs {
 
@@ -151,58 +152,11 @@ __global__ void __launch_bounds__(TEAM > 256 ? TEAM : 256) k_sh_fp32(const __gri
         }
         for (int sl = 0; sl < n_sl; ++sl) {
             if (a.project) {
-                // this subaperture's OPD straight from the screens: the arithmetic of the projection
-                // kernel (layer offsets in FP64, bilinear samples summed over the layers in order);
-                // a slice sees the layers through its own cone (the scale), the offsets are shared
                 const InstDesc &I = a.inst[W.inst];
-                const int L = proj_layers(I, D);
-                const int S = I.S;
-                const bool pow2 = (S & (S - 1)) == 0;
-                const int id = __ldg(W.subap + v), sy = id / W.n_sub, sx = id - sy * W.n_sub;
-                const float half = 0.5f * (float)(W.n_sub * n - 1);
-                float *out = D.opd + W.opd_off + (size_t)v * nn;
-                // the slice's geometric term 1/2 |x - r_L|^2 k_s relative to the subaperture centre r_b:
-                // k_s ((x - r_b).(r_b - r_L) + 1/2 |x - r_b|^2)
-                float ebx = 0.0f, eby = 0.0f, dxp = 0.0f, ks = 0.0f;
+                self_project(a, W, I, D, SD, sl, v, n, lo, tid, TEAM, so);
                 if (SD) {
-                    dxp = (float)(W.pupil_dx_over_ds * I.ds);
-                    const float c0 = 0.5f * (float)(n - 1);
-                    ebx = ((float)(sx * n) + c0 - half) * dxp - (float)W.launch_x;
-                    eby = ((float)(sy * n) + c0 - half) * dxp - (float)W.launch_y;
-                    ks = SD->k[sl];
-                }
-                for (int i = tid; i < nn; i += TEAM) {
-                    const int pp = i / n, qq = i - pp * n;
-                    const float xr = (float)(sx * n + qq) - half, yr = (float)(sy * n + pp) - half;
-                    float acc = 0.0f;
-                    for (int l = 0; l < L; ++l) {
-                        const LayerOffs L0 = lo[l];
-                        const float ch = SD ? SD->c[sl][l].x : L0.c, cl = SD ? SD->c[sl][l].y : L0.cl;
-                        int ou, ov, i0, i1, j0, j1;
-                        float fx, gy;
-                        screen_offset(ch, cl, L0.fu, xr, ou, fx);
-                        screen_offset(ch, cl, L0.fv, yr, ov, gy);
-                        wrap_pair(L0.bu + ou, S, pow2, i0, i1);
-                        wrap_pair(L0.bv + ov, S, pow2, j0, j1);
-                        if (!guard(i0 >= 0 && i1 < S && i1 >= 0 && j0 >= 0 && j1 < S && j1 >= 0 && i0 < S && j0 < S,
-                                   a.status))
-                            continue;
-                        const float *scr = layer_screen(I, D, l);
-                        const float *r0 = scr + (size_t)j0 * S, *r1 = scr + (size_t)j1 * S;
-                        const float s00 = __ldg(r0 + i0), s01 = __ldg(r0 + i1);
-                        const float s10 = __ldg(r1 + i0), s11 = __ldg(r1 + i1);
-                        const float top = fmaf(fx, s01 - s00, s00);
-                        const float bot = fmaf(fx, s11 - s10, s10);
-                        acc += fmaf(gy, bot - top, top);
-                    }
-                    if (W.uplink) acc += fmaf(W.uplink->x, xr, W.uplink->y * yr);
-                    if (sl == 0) out[i] = acc;
-                    if (SD) {
-                        const float ux = ((float)qq - 0.5f * (float)(n - 1)) * dxp;
-                        const float uy = ((float)pp - 0.5f * (float)(n - 1)) * dxp;
-                        acc += ks * fmaf(ux, ebx, fmaf(uy, eby, 0.5f * fmaf(ux, ux, uy * uy)));
-                    }
-                    so[i] = acc;
+                    const SliceTerm term(I, W, v, n);
+                    for (int i = tid; i < nn; i += TEAM) so[i] += term.at(SD->k[sl], i / n, i - (i / n) * n);
                 }
                 team_sync<TEAM>(team);
             }
@@ -369,14 +323,14 @@ cudaError_t generic_shape(const ShArgs &a, LaunchShape *out) {
 }
 }  // namespace
 
-cudaError_t n32_launch_shape(const ShArgs &a, LaunchShape *out);
+cudaError_t row_launch_shape(const ShArgs &a, LaunchShape *out);
 cudaError_t tc_launch_shape(const ShArgs &a, LaunchShape *out, bool f16);
 cudaError_t tc64_launch_shape(const ShArgs &a, LaunchShape *out, bool f16);
 
 cudaError_t spot_launch_shape(int kind, const ShArgs &a, LaunchShape *out) {
     switch (kind) {
         case kSpotGeneric: return generic_shape(a, out);
-        case kSpotN32: return n32_launch_shape(a, out);
+        case kSpotRow: return row_launch_shape(a, out);
         case kSpotTc: return a.N == 64 ? tc64_launch_shape(a, out, false) : tc_launch_shape(a, out, false);
         case kSpotTcF16: return a.N == 64 ? tc64_launch_shape(a, out, true) : tc_launch_shape(a, out, true);
         default: return cudaErrorInvalidValue;
@@ -506,23 +460,8 @@ __global__ void __launch_bounds__(256) k_noise(const float *E, int n, float ron,
         if (in0) e.x = E[i];
         if (in1) e.y = E[i + 1];
     }
-    const PairStream q = pair_stream(seed, pixel0 + (uint32_t)(in0 ? i : i + 1), wfs, tlo, thi);
-    const uint4 r = q.block(0);
-    float ze, zo;
-    box_muller_pair(r.x, r.y, ze, zo);
-    const float2 em = make_float2(inversion_mean(e.x), inversion_mean(e.y));
-    int k0, k1;
-    poisson_inversion_pair(em, make_float2(philox_unit(r.z), philox_unit(r.w)),
-                           make_float2(expf(-em.x), expf(-em.y)), rk2, k0, k1);
-    for (int s = 0; s < 2; ++s) {  // one PTRS call site
-        const float es = s ? e.y : e.x;
-        if (es >= 16.0f) {
-            const int k = poisson_ptrs(es, q, s);
-            if (s) k1 = k;
-            else k0 = k;
-        }
-    }
-    const float2 c = make_float2((float)k0 + ron * ze, (float)k1 + ron * zo);
+    float2 c;
+    noise_pair(e.x, e.y, ron, seed, pixel0 + (uint32_t)(in0 ? i : i + 1), wfs, tlo, thi, rk2, c.x, c.y);
     if (vec && in0 && in1) {
         *reinterpret_cast<float2 *>(C + i) = c;
     } else {

@@ -149,6 +149,9 @@ __device__ __forceinline__ void poisson_inversion_pair(float2 E, float2 u, float
     k1 = c1;
 }
 
+// The mean of an inversion search: E where the search applies, 0 (no draw) elsewhere.
+__device__ __forceinline__ float inversion_mean(float E) { return E > 0.0f && E < 16.0f ? E : 0.0f; }
+
 // PTRS for E >= 16: draws word 2 + parity of block 0, then blocks 1 + parity, 3 + parity,
 // ...  Rare for the workloads here, so it recomputes block 0 rather than keep it live.
 // Inlined: callers give it a single call site (an out-of-line call would make every live
@@ -197,6 +200,31 @@ __device__ __forceinline__ int poisson_count(float E, float u, float p0, const P
     return poisson_ptrs(E, q, parity);
 }
 
+// Both pixels of a generator pair (ee, eo: their means; pixel: either index), on every lane of a
+// converged warp; a pixel that is not wanted takes mean 0 and its result is dropped.
+__device__ __forceinline__ void noise_pair(float ee, float eo, float read_noise, uint64_t seed, uint32_t pixel,
+                                           uint32_t wfs, uint32_t tlo, uint32_t thi, const float4 *rk2, float &ce,
+                                           float &co) {
+    const PairStream q = pair_stream(seed, pixel, wfs, tlo, thi);
+    const uint4 r = q.block(0);
+    float ze, zo;
+    box_muller_pair(r.x, r.y, ze, zo);
+    const float2 em = make_float2(inversion_mean(ee), inversion_mean(eo));
+    int k0, k1;
+    poisson_inversion_pair(em, make_float2(philox_unit(r.z), philox_unit(r.w)), make_float2(expf(-em.x), expf(-em.y)),
+                           rk2, k0, k1);
+    for (int s = 0; s < 2; ++s) {  // one PTRS call site
+        const float es = s ? eo : ee;
+        if (es >= 16.0f) {
+            const int k = poisson_ptrs(es, q, s);
+            if (s) k1 = k;
+            else k0 = k;
+        }
+    }
+    ce = (float)k0 + read_noise * ze;
+    co = (float)k1 + read_noise * zo;
+}
+
 // One detector pixel: Poisson photon count plus Gaussian read noise (forms its pair's block).
 __device__ __forceinline__ float noise_pixel(float E, float read_noise, uint64_t seed,
                                              uint32_t pixel, uint32_t wfs, uint32_t tlo,
@@ -209,9 +237,6 @@ __device__ __forceinline__ float noise_pixel(float E, float read_noise, uint64_t
     const int k = poisson_count(E, philox_unit(parity ? r.w : r.z), expf(-E), q, parity);
     return (float)k + read_noise * (parity ? zo : ze);
 }
-
-// The mean of an inversion search: E where the search applies, 0 (no draw) elsewhere.
-__device__ __forceinline__ float inversion_mean(float E) { return E > 0.0f && E < 16.0f ? E : 0.0f; }
 
 // Fills rk2[i], i < kRecipTable / 2, with RN(1/k) twice for k = 2i + 1 and twice for 2i + 2; call
 // from every thread of the block.

@@ -286,7 +286,7 @@ extern "C" wfs_status wfs_measure_one_static(const wfs_telescope *tel, const wfs
     h_sa.status = (int *)(base + o_status);
     h_sa.n_inst = 1;
     h_sa.dyn[0] = dyn;
-    const int kind = sh_n32_supported(n, N, nd) ? kSpotN32 : kSpotGeneric;
+    const int kind = sh_row_supported(n, N) ? kSpotRow : kSpotGeneric;
     if ((e = launch_spot(kind, h_sa, s)) != cudaSuccess)
         return st_fail(WFS_ECUDA, "wfs_measure_one_static: spot launch");
     return WFS_OK;
