@@ -63,9 +63,11 @@ typedef enum {
 } wfs_status;
 
 /*
- * DFT arithmetic of a geometry (the rest of the path is FP32 throughout).  The two
- * tensor-core forms are built for n_fft = 32 with (n_pix_sub, n_det) = (10, 16) or
- * (8, 16); other geometries with them get WFS_EUNSUPPORTED from wfs_create.
+ * DFT arithmetic of a geometry (the rest of the path is FP32 throughout).  The two tensor-core
+ * forms are accepted for (n_pix_sub, n_fft, n_det) = (10, 32, 16), (8, 32, 16), (8, 16, 8),
+ * (6, 24, 12) and, NGS only, (32, 64, 32); other geometries with them get WFS_EUNSUPPORTED from
+ * wfs_create.  They name the least accurate arithmetic a geometry may run: the 16- and 24-point
+ * sensors run in FP32 with any of the three, which is both faster and more accurate there.
  */
 enum {
     WFS_PREC_FP32 = 0,    /* plain FP32 on the CUDA cores */
@@ -304,7 +306,10 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
  */
 wfs_status wfs_batch_tune(wfs_batch b, const float *const *screens, const double *t_s,
                           float *const *slopes_out, void *stream);
-/* Kernel classes of a batch (kind: 0 generic FP32, 1 FP32 N = 32, 2 tensor-core BF16x3). */
+/*
+ * Kernel classes of a batch (kind: 0 generic FP32, 1 FP32 with a warp per subaperture, 2 tensor-core
+ * BF16x3, 3 tensor-core FP16).
+ */
 typedef struct {
     int kind, n_pix_sub, n_fft, n_det, n_wfs, n_subaps, grid_cap, cta_warps;
 } wfs_batch_class;

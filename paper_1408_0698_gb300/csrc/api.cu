@@ -81,9 +81,21 @@ struct SpotGroup {
     int sl_count = 0, sl_blocks = 0;
 };
 
+// The geometries a tensor-core precision is accepted for: those with a tensor-core kernel, and the
+// configured 16- and 24-point sensors.
+bool tc_precision_supported(int n, int N, int nd) {
+    return sh_tc_supported(n, N, nd) || (N == 16 && n == 8 && nd == 8) || (N == 24 && n == 6 && nd == 12);
+}
+
+// Whether a geometry of a tensor-core precision runs a tensor-core kernel.  16- and 24-point DFTs run
+// in FP32 instead, which is the more accurate and the faster form: on the MMAs' 32-row tiles half or a
+// quarter of the rows are padding and the operands' splits, stores and two round trips remain (spot
+// kernel of 5,056 subapertures of n = 6, N = 24: 22.6 us against 29.2 us; 316 of n = 8, N = 16:
+// 10.5 against 12.6 us).
+bool runs_tc(const wfs_geometry &g) { return g.precision != WFS_PREC_FP32 && g.n_fft >= 32; }
+
 int spot_kind(const wfs_geometry &g) {
-    if (g.precision == WFS_PREC_BF16X3) return kSpotTc;
-    if (g.precision == WFS_PREC_FP16S) return kSpotTcF16;
+    if (runs_tc(g)) return g.precision == WFS_PREC_BF16X3 ? kSpotTc : kSpotTcF16;
     return sh_row_supported(g.n_pix_sub, g.n_fft) ? kSpotRow : kSpotGeneric;
 }
 
@@ -939,7 +951,7 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
         for (int w = 0; w < n_gs; ++w) lgs |= gs[w].geometry_index == i && gs[w].is_lgs;
         if (sh_tc64_supported(g.n_pix_sub, g.n_fft, g.n_det)) {
             if (lgs) return fail(nullptr, WFS_EUNSUPPORTED, who + " with n_fft = 64 is built for NGS sensors only");
-        } else if (!sh_tc_supported(g.n_pix_sub, g.n_fft, g.n_det)) {
+        } else if (!tc_precision_supported(g.n_pix_sub, g.n_fft, g.n_det)) {
             return fail(nullptr, WFS_EUNSUPPORTED,
                         who + " is built for (n_pix_sub, n_fft, n_det) = (10, 32, 16), (8, 32, 16), (8, 16, 8), "
                               "(6, 24, 12) and (32, 64, 32) (NGS)");
@@ -975,7 +987,7 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
             delete h;
             return cuda_fail(nullptr, e, "table upload");
         }
-        if (geom[i].precision == WFS_PREC_BF16X3 || geom[i].precision == WFS_PREC_FP16S) {
+        if (runs_tc(geom[i])) {
             const int n = geom[i].n_pix_sub, N = geom[i].n_fft;
             std::vector<uint8_t> b1, b2h, b2l, a0;
             if (N == 64)

@@ -1,7 +1,7 @@
 // k_sh_tc.cu -- the spot kernel with the DFT contraction on the 5th-generation
 // tensor cores (tcgen05, BF16 hi/lo split with three products, FP32
 // accumulation in tensor memory; or the same with FP16 hi/lo and per-subaperture
-// power-of-two operand scaling), for 32-point DFT geometries with n <= 10.
+// power-of-two operand scaling), for 32-point DFT geometries (n = 8 or 10, 16 x 16 detector).
 //
 // Arithmetic (Sec. 4 LGS SH: spot by DFT, sodium elongation, binning, noise,
 // centroid) is that of k_sh.cu; only the two contractions whose second operand
@@ -117,10 +117,8 @@ __device__ __forceinline__ void field_rows(const float2 *Fk, const float4 *X4, i
 
 template <int n, int N_, int nd, bool kSlices = false, bool kMmaU = false, int WG = kWG>
 struct TcLayout {
-    static constexpr int N = N_, D2 = 2 * n - 1, no = n | 1;
-    // N = 32 with a 16 x 16 detector: the elongation stage as a DFT across the 32 lanes and
-    // the noise in its own pass; other sizes: the stages as direct sums over the warp's rows
-    static constexpr bool kLane = N == 32 && nd == 16;
+    static constexpr int N = N_, D2 = 2 * n - 1;
+    static_assert(N == 32 && nd == 16, "one DFT row per lane, the lane DFT and the detector tile of spot_tail.cuh");
     // byte offsets; tensor-core tiles first (1024-aligned)
     static constexpr int oB1 = 0;                  // 64 rows x 128 B: [F_hi; F_hi; F_lo] blocks
     static constexpr int oB2h = oB1 + 8192;        // 32 rows x 128 B: [Ga_hi; Ga_hi]
@@ -135,22 +133,15 @@ struct TcLayout {
     static constexpr int oTab = oA + 16384 * WG;  // CUDA-core tables (float2)
     static constexpr int tFk = 0;                  // [p][k]  F[k][p] (U = F X on the CUDA cores)
     static constexpr int tFft = tFk + (kMmaU ? 0 : n * N);  // lane-DFT twiddles and phases (tail::fill_fft_table)
-    static constexpr int tG = tFft + (kLane ? tail::kFftTable : 0);  // [d][nd] G[d][i]
-    static constexpr int tGa = tG + n * nd;        // [d][k] Ga (direct-sum stages only)
-    static constexpr int tEnd = tGa + (kLane ? 0 : n * N);
+    static constexpr int tG = tFft + tail::kFftTable;  // [d][nd] G[d][i]
+    static constexpr int tEnd = tG + n * nd;
     static constexpr int oWarp = (oTab + tEnd * 8 + 15) / 16 * 16;  // per-warp scratch (float2)
     static constexpr int even(int x) { return (x + 1) & ~1; }
-    // 32-lane path: the NGS image rows (wI) alias the LGS scratch (wQ); X and Q hold column
+    // the NGS image rows (wI, [N][N + 1] floats) alias the LGS scratch (wQ); X and Q hold column
     // pairs, 16-byte aligned
-    static constexpr int wX = 0, wQ = wX + n * n;
-    // direct-sum path: Ta [N][no] over the consumed field X, then M [D2][n], P [D2][nd], B
-    // [nd][nd] floats; an NGS's image rows [N][N + 1] floats over X, then B
-    static constexpr int wTa = 0, wMg = even(n * n > N * no ? n * n : N * no), wP = wMg + D2 * n,
-                         wB = kLane ? 0 : wP + D2 * nd;
-    static constexpr int wI = kLane ? wQ : 0, wBn = even((N * (N + 1) + 1) / 2);
+    static constexpr int wX = 0, wQ = wX + n * n, wI = wQ;
     static_assert(wQ % 2 == 0, "16-byte aligned column-pair scratch");
-    static constexpr int lgs_end = kLane ? wQ + nd * n : even(wB + (nd * nd + 1) / 2);
-    static constexpr int ngs_end = kLane ? wI + (N * (N + 1) + 1) / 2 : wBn + (nd * nd + 1) / 2;
+    static constexpr int lgs_end = wQ + nd * n, ngs_end = wI + (N * (N + 1) + 1) / 2;
     // an LGS subaperture's elongation table K~ ([2n-1][n] complex), staged by cp.async at the
     // top of a group and read by the elongation stage; it may overlap the NGS rows, which an LGS
     // subaperture never writes (a warp's copies land before its next NGS image)
@@ -174,13 +165,12 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     constexpr int kWG = WG, kTcThreads = 128 * WG;
     constexpr uint32_t kTmemCols = 128 * WG;
     using E = TcElt<kF16>;
-    constexpr bool kLane = Lay::kLane;
     constexpr int D2 = Lay::D2, nd2 = nd * nd;
     static_assert(6 * n <= 64 && n <= 16, "the split DFT operand must fit one 64-element K atom");
     static_assert(N <= 32 && N >= 2 * n - 1, "one DFT row per lane; the autocorrelation fits the grid");
     static_assert(n % 2 == 0 && Lay::wKt % 2 == 0 && Lay::warp % 2 == 0 && Lay::oWarp % 16 == 0,
                   "16-byte aligned K~ staging");
-    static_assert(!kLane || nd2 % 32 == 0, "detector tile must split evenly over a warp");
+    static_assert(nd2 % 32 == 0, "detector tile must split evenly over a warp");
     static_assert(N % nd == 0 && nd % 2 == 0, "whole binning blocks; even detector rows");
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sB1 = smem + Lay::oB1, *sB2h = smem + Lay::oB2h, *sB2l = smem + Lay::oB2l;
@@ -189,7 +179,6 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     uint8_t *sA1 = smem + Lay::oA + 16384 * wg, *sA2 = sA1, *sB0 = sA1, *sA0 = smem + Lay::oA0;
     float2 *tab = reinterpret_cast<float2 *>(smem + Lay::oTab);
     float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft, *Gt = tab + Lay::tG;
-    float2 *Gat = tab + Lay::tGa;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + 32 * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 20);  // next group (dynamic split)
@@ -219,9 +208,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
                 Fk[p * N + k] = a.F[i];  // F[q*N + m] = F[m][q]: row index = p, column = k
             }
         }
-        if constexpr (kLane) tail::fill_fft_table<n>(fft, tid, kTcThreads);
-        else
-            for (int i = tid; i < n * N; i += kTcThreads) Gat[i] = a.Ga[i];
+        tail::fill_fft_table<n>(fft, tid, kTcThreads);
         for (int i = tid; i < n * nd; i += kTcThreads) Gt[i] = a.G[i];
     }
     if (wib == 0) {
@@ -534,36 +521,14 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         __syncwarp();
 
         // remaining stages on the CUDA cores (per warp)
-        if constexpr (kLane) {
-            float Bv[nd / 2];
-            if (W.is_lgs) {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                __syncwarp();
-                tail::lgs_binned<n, nd>(T, reinterpret_cast<float4 *>(Qw), fft, Gt,
-                                        Kts, lane, Bv);
-            } else
-                tail::ngs_binned<nd>(Iw, lane, Bv);
-            tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
-        } else {
-            float2 *wbase = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp;
-            float *Bw;
-            if (W.is_lgs) {
-                float2 *Ta = wbase + Lay::wTa;
-                if (lane < N) {
-#pragma unroll
-                    for (int d = 0; d < n; ++d) Ta[lane * Lay::no + d] = T[d];
-                }
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                __syncwarp();
-                Bw = reinterpret_cast<float *>(wbase + Lay::wB);
-                tail::lgs_direct<n, N, nd>(Ta, wbase + Lay::wMg, wbase + Lay::wP, Bw, Kts, Gat, Gt, lane);
-            } else {
-                __syncwarp();
-                Bw = reinterpret_cast<float *>(wbase + Lay::wBn);
-                tail::ngs_direct<N, nd>(Iw, Bw, lane);
-            }
-            tail::finish_direct<nd>(Bw, W, D, a.inst[W.inst].seed, v, lane);
-        }
+        float Bv[nd / 2];
+        if (W.is_lgs) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            tail::lgs_binned<n, nd>(T, reinterpret_cast<float4 *>(Qw), fft, Gt, Kts, lane, Bv);
+        } else
+            tail::ngs_binned<nd>(Iw, lane, Bv);
+        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy outlives the CTA
     fence_before_sync();
@@ -1012,12 +977,8 @@ cudaError_t shape_tc_k(const ShArgs &a, LaunchShape *out) {
 // ShArgs::mma_u the variant with U = F X as an MMA.
 template <int n, int N, int nd>
 cudaError_t shape_tc(const ShArgs &a, LaunchShape *out, bool f16) {
-    if constexpr (N == 32 && nd == 16) {
-        if (a.slice_opd_stride > 0)
-            return f16 ? shape_tc_k<n, N, nd, true, true, false>(a, out) : shape_tc_k<n, N, nd, true, false, false>(a, out);
-    } else {
-        if (a.slice_opd_stride > 0) return cudaErrorInvalidValue;
-    }
+    if (a.slice_opd_stride > 0)
+        return f16 ? shape_tc_k<n, N, nd, true, true, false>(a, out) : shape_tc_k<n, N, nd, true, false, false>(a, out);
     if (a.mma_u)
         return f16 ? shape_tc_k<n, N, nd, false, true, true>(a, out) : shape_tc_k<n, N, nd, false, false, true>(a, out);
     // ShArgs::cta_warps = 4: one warpgroup per CTA (else two)
@@ -1028,14 +989,8 @@ cudaError_t shape_tc(const ShArgs &a, LaunchShape *out, bool f16) {
 
 }  // namespace
 
-// The geometries with a tensor-core spot kernel: 32-point DFTs with a 16 x 16 detector (n = 8
-// or 10), and the other DFT sizes of the configured sensors -- 16-point (n = 8, 8 x 8
-// detector) and 24-point (n = 6, 12 x 12 detector).
-bool sh_tc_supported(int n, int N, int nd) {
-    return (N == 32 && nd == 16 && (n == 10 || n == 8)) || (N == 16 && n == 8 && nd == 8) ||
-           (N == 24 && n == 6 && nd == 12);
-}
-
+// The geometries with this kernel: 32-point DFTs with a 16 x 16 detector (n = 8 or 10).
+bool sh_tc_supported(int n, int N, int nd) { return N == 32 && nd == 16 && (n == 10 || n == 8); }
 // The per-slice LGS variant exists for the 32-point tensor-core geometries.
 bool sh_tc_slices_supported(int n, int N, int nd) { return N == 32 && nd == 16 && (n == 10 || n == 8); }
 
@@ -1106,8 +1061,6 @@ void build_tc_tiles(int n, int N, const double *F_re64, const double *F_im64, co
 cudaError_t tc_launch_shape(const ShArgs &a, LaunchShape *out, bool f16) {
     if (a.N == 32 && a.n == 10 && a.nd == 16) return shape_tc<10, 32, 16>(a, out, f16);
     if (a.N == 32 && a.n == 8 && a.nd == 16) return shape_tc<8, 32, 16>(a, out, f16);
-    if (a.N == 16 && a.n == 8 && a.nd == 8) return shape_tc<8, 16, 8>(a, out, f16);
-    if (a.N == 24 && a.n == 6 && a.nd == 12) return shape_tc<6, 24, 12>(a, out, f16);
     return cudaErrorInvalidValue;
 }
 
