@@ -60,6 +60,7 @@ struct GeomDev {
     int mask_words = 0;
     float2 *F = nullptr, *Ga = nullptr, *G = nullptr;
     uint8_t *tcB1 = nullptr, *tcB2h = nullptr, *tcB2l = nullptr;  // BF16X3 operand tiles
+    float4 Gc[kMaxUniG] = {};                                     // ShArgs::Gc
     uint8_t *tcA0 = nullptr;                                        // first-stage operand tile
 };
 
@@ -533,6 +534,7 @@ void fill_geom_args(ShArgs &sa, const GeomDev &G) {
     sa.mma_u = (mu && mu[0] == '1') ? 1 : 0;
     sa.tc_B2h = G.tcB2h;
     sa.tc_B2l = G.tcB2l;
+    memcpy(sa.Gc, G.Gc, sizeof sa.Gc);
 }
 
 const char *kind_name(int kind) {
@@ -988,7 +990,13 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
             return cuda_fail(nullptr, e, "table upload");
         }
         if (runs_tc(geom[i])) {
-            const int n = geom[i].n_pix_sub, N = geom[i].n_fft;
+            const int n = geom[i].n_pix_sub, N = geom[i].n_fft, nd = geom[i].n_det;
+            if (N == 32)
+                for (int ix = 0; ix < nd / 2; ++ix)
+                    for (int c = 0; c < n / 2; ++c) {
+                        const float2 g0 = Gb[(size_t)(2 * c) * nd + ix], g1 = Gb[(size_t)(2 * c + 1) * nd + ix];
+                        G.Gc[ix * (n / 2) + c] = make_float4(g0.x, g1.x, -g0.y, -g1.y);
+                    }
             std::vector<uint8_t> b1, b2h, b2l, a0;
             if (N == 64)
                 build_tc64_tiles(F64.data(), F64.data() + (size_t)n * N, geom[i].precision == WFS_PREC_FP16S, a0, b1);

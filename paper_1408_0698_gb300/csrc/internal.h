@@ -27,6 +27,7 @@ constexpr int kMaxNaSlices = 16;
 constexpr int kMaxN = 64;           // largest DFT size
 constexpr int kMaxNPix = 32;        // largest subaperture side in pupil pixels
 constexpr int kMaxInstances = 64;   // instances per launch (batch size limit)
+constexpr int kMaxUniG = 40;         // 8 columns x 5 column pairs (n <= 10)
 
 struct InstDesc {                   // static per instance
     int n_layers, S;                // turbulent layers; mirror layers follow them (InstDyn::n_dm)
@@ -113,6 +114,9 @@ struct ShArgs {
     const void *tc_B1, *tc_B2h, *tc_B2l;  // BF16X3 operand tiles (pre-swizzled)
     const void *tc_A0;                    // F's rows, four times over: the first DFT stage's operand
     int mma_u;                            // tensor-core kernels: U = F X as an MMA too (GBWFS_TC_MMA_U=1)
+    float4 Gc[kMaxUniG];                  // 32-point tensor-core kernels: G for the detector columns
+                                          // ix < nd/2, entry ix (n/2) + c = columns dx = 2c, 2c + 1 as
+                                          // (re, re, -im, -im); read at uniform addresses
     const InstDesc *inst;
     const WfsDesc *wfs;  // this launch's WFS entries (subap_begin relative to them)
     int n_wfs, total;

@@ -22,6 +22,13 @@
 // memory and returns).  U = F X, the column transform, binning, photometry,
 // noise and the centroid run on the CUDA cores exactly as in the FP32 kernels.
 //
+// Bound: the shared-memory and load/store wavefronts with their latency (61 % of that pipe, 46 % issue at
+// 16 warps per SM; with 20 or 24 warps the same time, so it is the pipe).  G of the binning stage comes
+// from the kernel parameters, the rows of Q stay in registers, K~ goes from global memory to registers
+// under the second product and the field is written as whole 16-byte entries: 640 -> 558 wavefronts and
+// 1,684 -> 1,557 warp instructions per LGS subaperture, ELT frame (27,792 of them) 94.3 -> 88.8 us, the
+// same bits.
+//
 // CTA = two warpgroups (4 warps each); warp w of a warpgroup owns subaperture 4g + w of its
 // group g and its lane k owns DFT row k, which is also TMEM lane 32 w + k of both accumulators.
 //
@@ -52,13 +59,29 @@ constexpr int kWG = 2;                   // independent warpgroups per CTA
 constexpr int kTcThreads = 128 * kWG;
 constexpr uint32_t kTmemCols = 128 * kWG;  // per warpgroup: D1 columns [0, 64), D2 [64, 96)
 // The field X of one subaperture in the warp's scratch as column pairs: entry [p][q/2] holds
-// (re q, re q+1, im q, im q+1) of row p (q even).
-template <int n>
-__device__ __forceinline__ void store_field(float4 *X4, int i, float c, float s) {
-    const int p = i / n, q = i - p * n;
-    float *e = reinterpret_cast<float *>(X4 + p * (n / 2) + (q >> 1)) + (q & 1);
-    e[0] = c;
-    e[2] = s;
+// (re q, re q+1, im q, im q+1) of row p (q even).  A lane forms whole entries (the pixels 2i, 2i + 1),
+// so that they are written as 16-byte words.  opd(i): the sample of pixel i; ref: the piston.
+template <int n, typename F>
+__device__ __forceinline__ void field_pairs(float4 *X4, F opd, float ref, float k_phase, const uint32_t *mk, int lane) {
+    constexpr int kE = n * n / 2, kM = (kE + 31) / 32;
+    float o0[kM], o1[kM];
+    uint32_t mw[kM];
+#pragma unroll
+    for (int m = 0; m < kM; ++m) {  // all of the lane's loads first
+        const int i = min(lane + 32 * m, kE - 1);
+        o0[m] = opd(2 * i);
+        o1[m] = opd(2 * i + 1);
+        mw[m] = __ldg(mk + (i >> 4)) >> (2 * (i & 15));
+    }
+#pragma unroll
+    for (int m = 0; m < kM; ++m) {
+        const int i = lane + 32 * m;
+        float s0, c0, s1, c1;
+        field_phasor(k_phase * (o0[m] - ref), s0, c0);
+        field_phasor(k_phase * (o1[m] - ref), s1, c1);
+        const bool l0 = mw[m] & 1u, l1 = mw[m] & 2u;
+        if (i < kE) X4[i] = make_float4(l0 ? c0 : 0.0f, l1 ? c1 : 0.0f, l0 ? s0 : 0.0f, l1 ? s1 : 0.0f);
+    }
 }
 
 // U[q] = sum_p F[k][p] X[p][q] for this lane's DFT row k (lanes k >= N get zeros).  The rows k
@@ -133,22 +156,16 @@ struct TcLayout {
     static constexpr int oTab = oA + 16384 * WG;  // CUDA-core tables (float2)
     static constexpr int tFk = 0;                  // [p][k]  F[k][p] (U = F X on the CUDA cores)
     static constexpr int tFft = tFk + (kMmaU ? 0 : n * N);  // lane-DFT twiddles and phases (tail::fill_fft_table)
-    static constexpr int tG = tFft + tail::kFftTable;  // [d][nd] G[d][i]
-    static constexpr int tEnd = tG + n * nd;
+    static constexpr int tEnd = tFft + tail::kFftTable;
     static constexpr int oWarp = (oTab + tEnd * 8 + 15) / 16 * 16;  // per-warp scratch (float2)
     static constexpr int even(int x) { return (x + 1) & ~1; }
-    // the NGS image rows (wI, [N][N + 1] floats) alias the LGS scratch (wQ); X and Q hold column
-    // pairs, 16-byte aligned
-    static constexpr int wX = 0, wQ = wX + n * n, wI = wQ;
-    static_assert(wQ % 2 == 0, "16-byte aligned column-pair scratch");
-    static constexpr int lgs_end = wQ + nd * n, ngs_end = wI + (N * (N + 1) + 1) / 2;
-    // an LGS subaperture's elongation table K~ ([2n-1][n] complex), staged by cp.async at the
-    // top of a group and read by the elongation stage; it may overlap the NGS rows, which an LGS
-    // subaperture never writes (a warp's copies land before its next NGS image)
-    static constexpr int wKt = lgs_end;
-    static constexpr int base_warp = even(wKt + D2 * n > ngs_end ? wKt + D2 * n : ngs_end);
-    // per-slice variant: the summed spot rows use the NGS rows (wI; K~ is staged after them)
-    static constexpr int warp = base_warp;
+    // per warp: the field X (column pairs, 16-byte aligned); then an NGS's image rows (wI,
+    // [N][N + 1] floats) or the binned image (wB), over the consumed field, but for the per-slice
+    // variant, whose summed spot rows (wI) live across the slices' fields
+    static constexpr int wX = 0, wI = kSlices ? even(n * n) : 0, wB = wI;
+    static constexpr int i_end = wI + (N * (N + 1) + 1) / 2, b_end = wB + tail::kBScratch / 2;
+    static constexpr int warp = even(n * n > (i_end > b_end ? i_end : b_end) ? n * n : (i_end > b_end ? i_end : b_end));
+    static_assert(wB % 2 == 0, "16-byte aligned scratch");
     // per warpgroup: 2 mbarriers (0), flag (16), next group (20), the first-stage mbarrier (24);
     // per-slice variant: the slice counts of its 4 warps (32)
     static constexpr int misc = kSlices ? 48 : 32;
@@ -168,8 +185,8 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     constexpr int D2 = Lay::D2, nd2 = nd * nd;
     static_assert(6 * n <= 64 && n <= 16, "the split DFT operand must fit one 64-element K atom");
     static_assert(N <= 32 && N >= 2 * n - 1, "one DFT row per lane; the autocorrelation fits the grid");
-    static_assert(n % 2 == 0 && Lay::wKt % 2 == 0 && Lay::warp % 2 == 0 && Lay::oWarp % 16 == 0,
-                  "16-byte aligned K~ staging");
+    static_assert(n % 2 == 0 && Lay::warp % 2 == 0 && Lay::oWarp % 16 == 0, "16-byte aligned scratch");
+    static_assert((nd / 2) * (n / 2) <= kMaxUniG, "G's columns fit the kernel parameters");
     static_assert(nd2 % 32 == 0, "detector tile must split evenly over a warp");
     static_assert(N % nd == 0 && nd % 2 == 0, "whole binning blocks; even detector rows");
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -178,7 +195,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     const int wg = wib >> 2, wq = wib & 3;  // warpgroup, warp within it (= TMEM lane quarter)
     uint8_t *sA1 = smem + Lay::oA + 16384 * wg, *sA2 = sA1, *sB0 = sA1, *sA0 = smem + Lay::oA0;
     float2 *tab = reinterpret_cast<float2 *>(smem + Lay::oTab);
-    float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft, *Gt = tab + Lay::tG;
+    float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + 32 * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + 32 * wg + 20);  // next group (dynamic split)
@@ -209,7 +226,6 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
             }
         }
         tail::fill_fft_table<n>(fft, tid, kTcThreads);
-        for (int i = tid; i < n * nd; i += kTcThreads) Gt[i] = a.G[i];
     }
     if (wib == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -236,8 +252,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     constexpr uint32_t idesc0 = tc_idesc(128, 128, E::fmt);
 
     float4 *X4 = reinterpret_cast<float4 *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wX);
-    float2 *Qw = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wQ;
-    float2 *Kts = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wKt;
+    float *Bw = reinterpret_cast<float *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wB);
     float *Iw = reinterpret_cast<float *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wI);
     const int row = wq * 32 + lane;  // this thread's row of the MMA tiles and TMEM lane
     const int groups = (a.total + 3) / 4;
@@ -258,16 +273,6 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         const InstDyn &D = a.dyn[W.inst];
         const int v = active ? g - W.subap_begin : 0;
         active = active && guard(v >= 0 && v < W.n_valid, a.status);
-        if (active && W.is_lgs) {
-            // K~ of this subaperture: (2n-1) n complex = 16-byte chunks (n even)
-            const float4 *src = reinterpret_cast<const float4 *>(W.ktil + (size_t)v * (D2 * n));
-            for (int c = lane; c < D2 * n / 2; c += 32) {
-                const uint32_t dst = smem_u32(reinterpret_cast<float4 *>(Kts) + c);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + c) : "memory");
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-
         float2 U[n];
 #pragma unroll
         for (int q = 0; q < n; ++q) U[q] = make_float2(0.0f, 0.0f);
@@ -351,25 +356,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
             const float *opd = D.opd + W.opd_off + (size_t)v * (n * n);
             const uint32_t *mk = W.mask + (size_t)v * a.mask_words;
             const float ref = __ldg(opd);
-            // all of the lane's loads first (element i = lane + 32 m, mask word m)
-            constexpr int kFw = (n * n + 31) / 32;
-            float o[kFw];
-            uint32_t mw[kFw];
-#pragma unroll
-            for (int m = 0; m < kFw; ++m) {
-                o[m] = lane + 32 * m < n * n ? __ldg(opd + lane + 32 * m) : 0.0f;
-                mw[m] = __ldg(mk + m);
-            }
-#pragma unroll
-            for (int m = 0; m < kFw; ++m) {
-                const int i = lane + 32 * m;
-                if (i < n * n) {
-                    const bool lit = (mw[m] >> lane) & 1u;
-                    float s, c;
-                    field_phasor(W.k_phase * (o[m] - ref), s, c);
-                    store_field<n>(X4, i, lit ? c : 0.0f, lit ? s : 0.0f);
-                }
-            }
+            field_pairs<n>(X4, [&](int i) { return __ldg(opd + i); }, ref, W.k_phase, mk, lane);
             __syncwarp();
             field_rows<n, N>(Fk, X4, lane, U);  // DFT rows k >= N are zero
         }
@@ -490,6 +477,9 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         wg_sync();
         fence_after_sync();
         if (*sflag) break;
+        // K~ of this subaperture, in flight while the second product runs
+        float4 kq[n / 2];
+        if (active && W.is_lgs) tail::load_ktil<n>(W.ktil + (size_t)v * (D2 * n), lane, kq);
         if (issuer) {
 #pragma unroll
             for (int s = 0; s < 4; ++s)
@@ -523,14 +513,11 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         // remaining stages on the CUDA cores (per warp)
         float Bv[nd / 2];
         if (W.is_lgs) {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncwarp();
-            tail::lgs_binned<n, nd>(T, reinterpret_cast<float4 *>(Qw), fft, Gt, Kts, lane, Bv);
+            tail::lgs_binned<n, nd>(T, Bw, fft, a.Gc, kq, lane, Bv);
         } else
             tail::ngs_binned<nd>(Iw, lane, Bv);
         tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy outlives the CTA
     fence_before_sync();
     __syncthreads();
     if (*sflag && issuer && a.status) atomicCAS(a.status, 0, 5 /* WFS_ETIMEOUT */);
@@ -555,8 +542,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
     using E = TcElt<kF16>;
     constexpr int N = 32, D2 = Lay::D2, nd2 = nd * nd;
     static_assert(6 * n <= 64 && n <= 16, "the split DFT operand must fit one 64-element K atom");
-    static_assert(n % 2 == 0 && Lay::wKt % 2 == 0 && Lay::warp % 2 == 0 && Lay::oWarp % 16 == 0,
-                  "16-byte aligned K~ staging");
+    static_assert(n % 2 == 0 && Lay::warp % 2 == 0 && Lay::oWarp % 16 == 0, "16-byte aligned scratch");
+    static_assert((nd / 2) * (n / 2) <= kMaxUniG, "G's columns fit the kernel parameters");
     static_assert(nd <= 32 && nd2 % 32 == 0, "detector tile must split evenly over a warp");
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sB1 = smem + Lay::oB1, *sB2h = smem + Lay::oB2h, *sB2l = smem + Lay::oB2l;
@@ -564,7 +551,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
     const int wg = wib >> 2, wq = wib & 3;  // warpgroup, warp within it (= TMEM lane quarter)
     uint8_t *sA1 = smem + Lay::oA + 16384 * wg, *sA2 = sA1;
     float2 *tab = reinterpret_cast<float2 *>(smem + Lay::oTab);
-    float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft, *Gt = tab + Lay::tG;
+    float2 *Fk = tab + Lay::tFk, *fft = tab + Lay::tFft;
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + Lay::misc * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 20);  // next group (dynamic split)
@@ -587,7 +574,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
             Fk[p * N + k] = a.F[i];  // F[q*N + m] = F[m][q]: row index = p, column = k
         }
         tail::fill_fft_table<n>(fft, tid, kTcThreads);
-        for (int i = tid; i < n * nd; i += kTcThreads) Gt[i] = a.G[i];
     }
     if (wib == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -612,8 +598,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
     constexpr uint32_t idesc1 = tc_idesc(128, 64, E::fmt), idesc2 = tc_idesc(128, 32, E::fmt);
 
     float4 *X4 = reinterpret_cast<float4 *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wX);
-    float2 *Qw = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wQ;
-    float2 *Kts = reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wKt;
+    float *Bw = reinterpret_cast<float *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wB);
     float *Iw = reinterpret_cast<float *>(reinterpret_cast<float2 *>(smem + Lay::oWarp) + wib * Lay::warp + Lay::wI);
     const int row = wq * 32 + lane;  // this thread's row of the MMA tiles and TMEM lane
     const int groups = (a.total + 3) / 4;
@@ -634,18 +619,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         const InstDyn &D = a.dyn[W.inst];
         const int v = active ? g - W.subap_begin : 0;
         active = active && guard(v >= 0 && v < W.n_valid, a.status);
-        // K~ of this subaperture: (2n-1) n complex = 16-byte chunks (n even); the per-slice
-        // variant stages it after its slices, whose summed rows share the space
-        auto stage_ktil = [&]() {
-            const float4 *src = reinterpret_cast<const float4 *>(W.ktil + (size_t)v * (D2 * n));
-            for (int c = lane; c < D2 * n / 2; c += 32) {
-                const uint32_t dst = smem_u32(reinterpret_cast<float4 *>(Kts) + c);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + c) : "memory");
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        if (!kSlices && active && W.is_lgs) stage_ktil();
-
         // slices: one for the elongation-kernel model; the warpgroup runs the largest count of
         // its four subapertures (a subaperture with fewer adds nothing in the extra ones)
         const SliceDesc *SD = (kSlices && active) ? W.slices : nullptr;
@@ -684,25 +657,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
                 };
                 const uint32_t *mk = W.mask + (size_t)v * a.mask_words;
                 const float ref = __ldg(opd) + geo(0);
-                // all of the lane's loads first (element i = lane + 32 m, mask word m)
-                constexpr int kFw = (n * n + 31) / 32;
-                float o[kFw];
-                uint32_t mw[kFw];
-#pragma unroll
-                for (int m = 0; m < kFw; ++m) {
-                    o[m] = lane + 32 * m < n * n ? __ldg(opd + lane + 32 * m) : 0.0f;
-                    mw[m] = __ldg(mk + m);
-                }
-#pragma unroll
-                for (int m = 0; m < kFw; ++m) {
-                    const int i = lane + 32 * m;
-                    if (i < n * n) {
-                        const bool lit = (mw[m] >> lane) & 1u;
-                        float s, c;
-                        field_phasor(W.k_phase * ((o[m] + geo(i)) - ref), s, c);
-                        store_field<n>(X4, i, lit ? c : 0.0f, lit ? s : 0.0f);
-                    }
-                }
+                field_pairs<n>(X4, [&](int i) { return __ldg(opd + i) + geo(i); }, ref, W.k_phase, mk, lane);
                 __syncwarp();
                 field_rows<n, N>(Fk, X4, lane, U);
             }
@@ -819,8 +774,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         if (quit) break;
         int ei = 0;  // FP16: the second operand carries 2^ei
         if (kSlices) {
-            // the summed rows -> second operand row [I_hi | I_lo] (after the last slice's MMA), then
-            // the K~ staging, which reuses their space
+            // the summed rows -> second operand row [I_hi | I_lo] (after the last slice's MMA)
             if constexpr (kF16) {
                 float mx = 0.0f;
 #pragma unroll
@@ -839,14 +793,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
                 *reinterpret_cast<uint4 *>(sA2 + sw128_off(row, c4 * 8)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
                 *reinterpret_cast<uint4 *>(sA2 + sw128_off(row, (4 + c4) * 8)) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
             }
-            __syncwarp();
-            if (active && W.is_lgs) stage_ktil();
         }
         fence_async_smem();
         fence_before_sync();
         wg_sync();
         fence_after_sync();
         if (*sflag) break;
+        // K~ of this subaperture, in flight while the second product runs
+        float4 kq[n / 2];
+        if (active && W.is_lgs) tail::load_ktil<n>(W.ktil + (size_t)v * (D2 * n), lane, kq);
         if (issuer) {
 #pragma unroll
             for (int s = 0; s < 4; ++s)
@@ -879,15 +834,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         // remaining stages on the CUDA cores (per warp)
         float Bv[nd / 2];
         if (W.is_lgs) {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncwarp();
-            tail::lgs_binned<n, nd>(T, reinterpret_cast<float4 *>(Qw), fft, Gt, Kts,
-                                    lane, Bv);
+            tail::lgs_binned<n, nd>(T, Bw, fft, a.Gc, kq, lane, Bv);
         } else
             tail::ngs_binned<nd>(Iw, lane, Bv);
         tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy outlives the CTA
     fence_before_sync();
     __syncthreads();
     if (*sflag && issuer && a.status) atomicCAS(a.status, 0, 5 /* WFS_ETIMEOUT */);

@@ -5,7 +5,7 @@
 //
 //   M[dy][dx] = Kt[dy][dx] sum_k Ga(dy, k) T[k][dx]       (k = lane: a 32-point DFT)
 //   Q[iy][dx] = sum_dy G(dy, iy) M[dy][dx]                 (an nd-point DFT over dy)
-//   B[iy][ix] = Re sum_dx Q[iy][dx] G[dx][ix]              (lane = ix, half-warp = iy half)
+//   B[iy][ix] = Re sum_dx Q[iy][dx] G[dx][ix]              (lane = iy, column half)
 // with Ga(dy, k) = exp(+2 pi i (k - cN) dy / N) = ph(dy) w^(k dy), w = exp(2 pi i / N),
 // ph(dy) = exp(-2 pi i cN dy / N), and G(dy, i) = sum_{r<b} exp(-2 pi i (b i + r - cN) dy / N)
 // (conjugated for dy < 0).  The sum over k is a DFT of each column across the lanes: radix 2,
@@ -16,8 +16,12 @@
 // M[dy][dx].  The lanes i and i ^ 1 hold the frequencies f and f + 16 (the same j, since
 // nd = 16), so one shuffle folds them, and the positions p = i >> 1 hold j = bitrev4(p): a
 // decimation-in-time DFT across the positions ends with Q[p] in natural order, the even lane
-// of each pair working the first column pairs and the odd lane the rest.  Then
-// E = photons fill B / sum B, C = Poisson(E) + ron z (or E), and the centre of gravity.
+// of each pair working the first column pairs and the odd lane the rest.  The lane pair then swaps
+// its halves, so that both lanes hold row p of Q, and the even lane forms the columns ix < nd/2 of
+// B, the odd lane their mirrors nd - 1 - ix: G(dx, nd-1-ix) = conj G(dx, ix), so every lane
+// multiplies by the same numbers, which come from the kernel's parameters (the constant port) and
+// not from shared memory.  Then E = photons fill B / sum B, C = Poisson(E) + ron z (or E), and the
+// centre of gravity.
 #pragma once
 #include "internal.h"
 #include "noise.cuh"
@@ -69,14 +73,27 @@ __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 
+// K~ of subaperture v for this lane's frequency: the entries its share of the elongation stage takes
+// (rows past the band read the nearest row and are multiplied by zero).
+template <int n>
+__device__ __forceinline__ void load_ktil(const float2 *kt, int lane, float4 (&kq)[n / 2]) {
+    const int f = (int)(__brev((unsigned)lane) >> 27), dy = f < 16 ? f : f - 32;
+    const int dyi = min(max(dy + n - 1, 0), 2 * n - 2);
+    const float4 *src = reinterpret_cast<const float4 *>(kt + dyi * n);  // n even: rows of 16-byte words
+#pragma unroll
+    for (int c = 0; c < n / 2; ++c) kq[c] = __ldg(src + c);
+}
+
+constexpr int kBScratch = 272;  // floats: the 16 x 16 image, its lower half 16 words off
+
 // T: this lane's row k = lane of the first stage (T[k][dx], dx < n), consumed.  fft: the
-// table above.  Gt: [n][nd] G[d][i].  kt: the subaperture's K~ [2n-1][n] (global or shared
-// memory).  Q is per-warp scratch ([nd][n/2], 16-byte aligned), each entry a column pair
-// (re dx, re dx+1, im dx, im dx+1).
+// table above.  kq: load_ktil.  Gc: uniform G for ix < nd/2, entry ix (n/2) + c holds the columns
+// dx = 2c, 2c + 1 as (re, re, -im, -im) (ShArgs::Gc).  Bs is per-warp scratch (kBScratch floats,
+// 16-byte aligned).
 // On return Bv[j] = B[half * nd/2 + j][ix] for lane = half * 16 + ix.
 template <int n, int nd>
-__device__ __forceinline__ void lgs_binned(float2 (&T)[n], float4 *Q, const float2 *fft, const float2 *Gt,
-                                           const float2 *kt, int lane, float (&Bv)[nd / 2]) {
+__device__ __forceinline__ void lgs_binned(float2 (&T)[n], float *Bs, const float2 *fft, const float4 *Gc,
+                                           const float4 (&kq)[n / 2], int lane, float (&Bv)[nd / 2]) {
     constexpr int P = n / 2, PH = (P + 1) / 2;
     static_assert(nd == 16, "the detector tile maps to 16 lanes x 2 half-warps");
     static_assert(n <= 16, "frequencies |dy| < n must be distinct modulo 32");
@@ -109,16 +126,13 @@ __device__ __forceinline__ void lgs_binned(float2 (&T)[n], float4 *Q, const floa
     // h(dy) M[dy] for the lane's frequency (zero outside the band |dy| < n, through the table),
     // then folded with the lane holding dy -/+ 16
     {
-        const int f = (int)(__brev((unsigned)lane) >> 27), dy = f < 16 ? f : f - 32;
-        const int dyi = min(max(dy + n - 1, 0), 2 * n - 2);
         const float2 ph = fft[5 * 32 + lane];
         const float2 phx = dup2(ph.x), phy = dup2(ph.y), nphy = dup2(-ph.y);
 #pragma unroll
         for (int c = 0; c < P; ++c) {
             const float2 xr = fma2(Ti[c], nphy, mul2(Tr[c], phx));
             const float2 xi = fma2(Ti[c], phx, mul2(Tr[c], phy));
-            const float2 k0 = kt[dyi * n + 2 * c], k1 = kt[dyi * n + 2 * c + 1];
-            const float2 kr = make_float2(k0.x, k1.x), ki = make_float2(k0.y, k1.y);
+            const float2 kr = make_float2(kq[c].x, kq[c].z), ki = make_float2(kq[c].y, kq[c].w);
             const float2 mr = fma2(xi, make_float2(-ki.x, -ki.y), mul2(xr, kr));
             const float2 mi = fma2(xi, kr, mul2(xr, ki));
             Tr[c] = __fadd2_rn(mr, make_float2(__shfl_xor_sync(0xffffffffu, mr.x, 1),
@@ -163,36 +177,57 @@ __device__ __forceinline__ void lgs_binned(float2 (&T)[n], float4 *Q, const floa
             Wi[j] = fma2(sg, vi, pi);
         }
     }
-    const int ix = lane & 15, half = lane >> 4;
-    __syncwarp();  // earlier reads of the scratch by other lanes are done
+    // row iy = lane >> 1 of Q in both lanes of the pair; the odd lane's columns are mirrored, which
+    // changes the sign of Im G: taken into Im Q
+    const float2 sgn = dup2(par ? -1.0f : 1.0f);
+    float2 qr[P], qi[P];
     {
-        const int iy = lane >> 1;
+        float2 pr[PH], pi[PH];
 #pragma unroll
         for (int j = 0; j < PH; ++j) {
-            const int c = par ? PH + j : j;
-            if (c < P) Q[iy * P + c] = make_float4(Wr[j].x, Wr[j].y, Wi[j].x, Wi[j].y);
+            Wi[j] = mul2(Wi[j], sgn);
+            pr[j] = make_float2(__shfl_xor_sync(0xffffffffu, Wr[j].x, 1), __shfl_xor_sync(0xffffffffu, Wr[j].y, 1));
+            pi[j] = make_float2(__shfl_xor_sync(0xffffffffu, Wi[j].x, 1), __shfl_xor_sync(0xffffffffu, Wi[j].y, 1));
+        }
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+            const int j = c < PH ? c : c - PH;
+            const bool mine = c < PH ? !par : par;
+            qr[c] = make_float2(mine ? Wr[j].x : pr[j].x, mine ? Wr[j].y : pr[j].y);
+            qi[c] = make_float2(mine ? Wi[j].x : -pi[j].x, mine ? Wi[j].y : -pi[j].y);
         }
     }
-    __syncwarp();
-    // B[iy][ix] for iy in this half: Re sum_dx Q[iy][dx] G[dx][ix], even and odd columns summed
-    // apart
-    float2 gcx[P], ngcy[P];
-#pragma unroll
-    for (int c = 0; c < P; ++c) {
-        const float2 g0 = Gt[(2 * c) * nd + ix], g1 = Gt[(2 * c + 1) * nd + ix];
-        gcx[c] = make_float2(g0.x, g1.x);
-        ngcy[c] = make_float2(-g0.y, -g1.y);
-    }
+    // B[iy][ix] = Re sum_dx Q[iy][dx] G[dx][ix], even and odd columns dx summed apart
+    float bt[nd / 2];
 #pragma unroll
     for (int j = 0; j < nd / 2; ++j) {
-        const int iy = half * (nd / 2) + j;
         float2 s = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int c = 0; c < P; ++c) {
-            const float4 qv = Q[iy * P + c];
-            s = fma2(make_float2(qv.x, qv.y), gcx[c], fma2(make_float2(qv.z, qv.w), ngcy[c], s));
+            const float4 g = Gc[j * P + c];
+            s = fma2(qr[c], make_float2(g.x, g.y), fma2(qi[c], make_float2(g.z, g.w), s));
         }
-        Bv[j] = s.x + s.y;
+        bt[j] = s.x + s.y;
+    }
+    // to lane = (row half, column): 16-byte words w of row iy at w ^ (bit 1 of iy), so that neither
+    // side meets a bank twice
+    const int iy = lane >> 1, sw = (iy >> 1) & 1;
+    float *row = Bs + iy * nd + (iy >= 8 ? 16 : 0);
+    __syncwarp();  // earlier reads of the scratch by other lanes are done
+    float4 *row4 = reinterpret_cast<float4 *>(row);
+    if (par) {
+        row4[3 ^ sw] = make_float4(bt[3], bt[2], bt[1], bt[0]);
+        row4[2 ^ sw] = make_float4(bt[7], bt[6], bt[5], bt[4]);
+    } else {
+        row4[0 ^ sw] = make_float4(bt[0], bt[1], bt[2], bt[3]);
+        row4[1 ^ sw] = make_float4(bt[4], bt[5], bt[6], bt[7]);
+    }
+    __syncwarp();
+    const int ix = lane & 15, half = lane >> 4;
+#pragma unroll
+    for (int j = 0; j < nd / 2; ++j) {
+        const int y = half * (nd / 2) + j;
+        Bv[j] = Bs[y * nd + half * 16 + ((((ix >> 2) ^ ((y >> 1) & 1)) << 2) | (ix & 3))];
     }
 }
 
