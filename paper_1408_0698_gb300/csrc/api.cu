@@ -70,7 +70,7 @@ struct SpotGroup {
     int first = 0, count = 0, total = 0;
     int kind = 0;            // SpotKind
     int grid_cap = 0, cta_warps = 0;
-    int proj_base = 0, proj_count = 0;  // this group's projection blocks
+    ProjRange proj_base{0, 0}, proj_count{0, 0};  // this group's projection blocks
     // LGS per-slice model: the group runs a per-slice spot kernel (the 32-point kernels' variants
     // after a projection of every (WFS, slice) pair, else the self-projecting generic kernel); the
     // kind and launch shape of the elongation-kernel model are kept to restore it
@@ -79,7 +79,8 @@ struct SpotGroup {
     // 32-point kernels: the per-slice OPDs come from one projection of every (WFS, slice) pair
     bool sl_projected = false;
     WfsDesc *d_sl_wfs = nullptr;
-    int sl_count = 0, sl_blocks = 0;
+    int sl_count = 0;
+    ProjRange sl_blocks{0, 0};
 };
 
 // The geometries a tensor-core precision is accepted for: those with a tensor-core kernel, and the
@@ -112,7 +113,7 @@ struct GsDev {
     float2 *d_ktil = nullptr;
     float2 *d_ktil_g = nullptr;  // per-slice model: the Gaussian extent alone
     int4 *d_segs = nullptr;
-    int n_segs = 0, seg_cols = 0, tiled = 0;
+    int n_segs = 0, n_full = 0, tiled = 0;
     double up_diam = 0.0;   // LGS uplink beam diameter (0: off)
     int up_n = 0;
     size_t slope_off = 0, opd_off = 0, int_off = 0, det_off = 0;
@@ -127,9 +128,7 @@ struct wfs_ctx {
     std::vector<WfsDesc> wfs_host;
     WfsDesc *d_wfs = nullptr;
     std::vector<SpotGroup> groups;
-    int proj_blocks = 0, proj_box = 0;
-    int proj_stage = 0;                 // bulk-copy projection box floats (-1: that form is off)
-    bool screens_host_mapped = false;   // the screens of the current call are mapped host memory
+    int proj_rows = 0;      // rows of the WFSs' largest projection box
     wfs_telescope tel{};
     std::vector<GeomDev> geoms;
     std::vector<GsDev> gs;
@@ -194,7 +193,8 @@ struct LoopDm {
 // (instance i = mode k of the chunk pushed (i = 2k) or pulled (i = 2k + 1)), each with its own
 // mirror layer, OPD, expected images and slopes.
 struct CalibScratch {
-    int gs = -1, kind = 0, geom = 0, group = 0, nv = 0, blocks_per_wfs = 0;
+    int gs = -1, kind = 0, geom = 0, group = 0, nv = 0;
+    ProjRange blocks_per_wfs{0, 0};
     size_t opd_stride = 0;
     WfsDesc *d_wfs = nullptr;        // [kMaxInstances]
     InstDesc *d_inst = nullptr;      // [n_dm][kMaxInstances]: a mirror as the only layer
@@ -241,9 +241,8 @@ struct wfs_batch_ctx {
     WfsDesc *d_wfs = nullptr;
     std::vector<WfsDesc> wfs_host;
     std::vector<BatchClass> classes;
-    int proj_blocks = 0, proj_box = 0;
-    int proj_stage = 0;                 // bulk-copy projection box floats (-1: that form is off)
-    int graph_stage = 0;                // the projection form the graph was built with
+    ProjRange proj_blocks{0, 0};
+    int proj_rows = 0;      // rows of the WFSs' largest projection box
     ProjArgs *pa = nullptr;          // parameter blocks the graph nodes point to
     std::vector<ShArgs *> sa;
     cudaGraph_t graph = nullptr;
@@ -278,23 +277,6 @@ wfs_status cuda_fail(wfs_handle h, cudaError_t e, const char *what) {
 }
 
 bool is_finite(double x) { return std::isfinite(x); }
-
-bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
-
-// The bulk-copy projection's box floats for WFS d on screens of side S: 0 for a WFS without
-// tiles, -1 where its boxes cannot move by bulk copies (rows not a whole number of 16-byte units,
-// or a box wider than the screen).
-int bulk_stage_floats(const WfsDesc &d, int S) {
-    if (!d.tiled) return 0;
-    if (S % 4 || d.seg_cols + 8 > S || d.n + 3 > S) return -1;
-    return project_stage_floats(d);
-}
-
-// Folds one WFS's value into a launch's: the largest box, or -1 once any WFS cannot use the form.
-void merge_stage(int &acc, int v) {
-    if (acc < 0 || v < 0) acc = -1;
-    else if (v > acc) acc = v;
-}
 
 constexpr size_t kMaxTimedLaunches = 65536;
 
@@ -577,22 +559,18 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
     cudaError_t e;
     pa.inst = h->d_inst;
     pa.n_inst = 1;
-    pa.box_cap = h->proj_box;
-    // the bulk-copy form reads 16-byte rows of device memory
-    pa.stage_cap = (h->proj_stage > 0 && !h->screens_host_mapped && aligned16(screens) &&
-                    (n_dm == 0 || aligned16(dm_layers)))
-                       ? h->proj_stage
-                       : 0;
+    pa.box_rows = h->proj_rows;
     pa.max_layers = h->inst_host.n_layers + n_dm;
     pa.status = h->d_status;
     pa.dyn[0] = dyn;
     // projection of a contiguous range of the WFS table (a group's WFSs, or all of them)
     auto project = [&](const SpotGroup &G, cudaStream_t ls) -> cudaError_t {
-        const int blocks = G.proj_count;
-        if (blocks <= 0) return cudaSuccess;
+        const ProjRange blocks = G.proj_count;
+        if (blocks.full + blocks.part <= 0) return cudaSuccess;
         pa.wfs = h->d_wfs + G.first;
         pa.n_wfs = G.count;
-        pa.block_base = G.proj_base;
+        pa.block_base = G.proj_base.full;
+        pa.part_base = G.proj_base.part;
         pa.work = h->d_work + 2 * (h->groups.size() + 1) + 2 * (&G - h->groups.data());
         long slot = timed_begin(h, "project", ls);
         cudaError_t err = launch_project(pa, blocks, ls, ls == stream && h->n_uplink > 0 && !h->timing);
@@ -670,7 +648,7 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         const bool fused = G.kind == kSpotGeneric || G.per_slice || (is_tc(G.kind) && geo.n_fft == 64) ||
                            (G.kind == kSpotRow && !(geo.n_fft == 32 && geo.n_det == 16));
         if (!fused && (e = project(G, ss)) != cudaSuccess) return cuda_fail(h, e, "projection launch");
-        if ((e = launch_group(G, ss, !fused && G.proj_count > 0, fused ? 1 : 0)) != cudaSuccess)
+        if ((e = launch_group(G, ss, !fused, fused ? 1 : 0)) != cudaSuccess)
             return cuda_fail(h, e, "spot launch");
         if ((e = cudaEventRecord(h->ev_join[k], ss)) != cudaSuccess) return cuda_fail(h, e, "join");
         ++k;
@@ -682,7 +660,7 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
             // then the 32-point kernel's per-slice variant
             pa.wfs = G.d_sl_wfs;
             pa.n_wfs = G.sl_count;
-            pa.block_base = 0;
+            pa.block_base = pa.part_base = 0;
             pa.work = h->d_work + 2 * (h->groups.size() + 1) + 2 * big;
             pa.dyn[0].opd = h->d_opd_sl;
             long slot = timed_begin(h, "project", stream);
@@ -705,10 +683,9 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
             if (G.total > 0 && (e = launch_group(G, stream, false, 2)) != cudaSuccess)
                 return cuda_fail(h, e, "spot launch");
         } else {
-            // with a single group this projects every WFS (blocks 0 .. proj_blocks)
             if ((e = project(G, stream)) != cudaSuccess)
                 return cuda_fail(h, e, "projection launch");
-            if (G.total > 0 && (e = launch_group(G, stream, G.proj_count > 0, 0)) != cudaSuccess)
+            if (G.total > 0 && (e = launch_group(G, stream, true, 0)) != cudaSuccess)
                 return cuda_fail(h, e, "spot launch");
         }
     }
@@ -755,7 +732,7 @@ wfs_status build_slice_projection(wfs_handle h) {
         G.d_sl_wfs = nullptr;
         if (!G.sl_projected) continue;
         std::vector<WfsDesc> t;
-        int blocks = 0;
+        ProjRange blocks{0, 0};
         for (int q = 0; q < G.count; ++q) {
             const WfsDesc &d0 = h->wfs_host[G.first + q];
             const GsDev &gd = h->gs[d0.gs_index];
@@ -764,8 +741,7 @@ wfs_status build_slice_projection(wfs_handle h) {
                 WfsDesc d = d0;
                 if (d0.is_lgs) d.range_m = gd.na_alt[sl];
                 d.opd_off = d0.opd_off + (long long)(sl * h->opd_total);
-                d.proj_block_begin = blocks;
-                blocks += project_blocks(d);
+                place_blocks(d, blocks);
                 t.push_back(d);
             }
         }
@@ -871,7 +847,8 @@ wfs_status calib_prepare(wfs_loop lp, int gs) {
         w[i].inst = i;
         w[i].opd_off = w[i].slope_off = w[i].int_off = w[i].det_off = 0;
         w[i].uplink = nullptr;  // no turbulence: no uplink tilt
-        w[i].proj_block_begin = i * c.blocks_per_wfs;
+        w[i].proj_block_begin = i * c.blocks_per_wfs.full;
+        w[i].proj_part_begin = i * c.blocks_per_wfs.part;
         w[i].subap_begin = i * c.nv;
     }
     const int n_dm = (int)lp->dms.size();
@@ -1064,10 +1041,8 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
         s.tiled = (tel->diameter_m / Np) / layers->screen_dx_m <= 1.0 + 1e-12 && s.n_valid > 0;
         if (s.tiled) {
             std::vector<int4> segs;
-            int run = 0;
-            build_segments(s.ids, g.n_sub, segment_max_count(n), segs, &run);
+            s.n_full = build_segments(s.ids, g.n_sub, n, segs);
             s.n_segs = (int)segs.size();
-            s.seg_cols = run * n;
             if ((e = upload(&s.d_segs, segs)) != cudaSuccess) {
                 release(h);
                 delete h;
@@ -1115,6 +1090,7 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
         I.n_layers = h->n_layers;
         I.S = h->S;
         I.ds = h->ds;
+        I.inv_ds = 1.0 / I.ds;
         for (int l = 0; l < h->n_layers; ++l) {
             I.alt[l] = h->alt[l];
             I.vx[l] = h->vx[l];
@@ -1123,7 +1099,7 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
             I.y0[l] = h->y0[l];
         }
         I.seed = seed;
-        int blocks = 0;
+        ProjRange blocks{0, 0};
         for (int gi = 0; gi < n_geom; ++gi) {
             SpotGroup G;
             G.geom = gi;
@@ -1159,24 +1135,21 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
                 d.det_off = (long long)s.det_off;
                 d.segs = s.d_segs;
                 d.n_segs = s.n_segs;
+                d.n_full = s.n_full;
                 d.tiled = s.tiled;
-                d.seg_cols = s.seg_cols;
                 d.launch_x = s.gs.launch_x_m;
                 d.launch_y = s.gs.launch_y_m;
                 d.uplink = nullptr;
-                d.proj_block_begin = blocks;
-                blocks += project_blocks(d);
-                if (project_box_floats(d) > h->proj_box) h->proj_box = project_box_floats(d);
-                merge_stage(h->proj_stage, bulk_stage_floats(d, h->S));
+                place_blocks(d, blocks);
+                h->proj_rows = std::max(h->proj_rows, project_box_rows(d));
                 d.subap_begin = G.total;
                 G.total += s.n_valid;
                 h->wfs_host.push_back(d);
                 ++G.count;
             }
-            G.proj_count = blocks - G.proj_base;
+            G.proj_count = {blocks.full - G.proj_base.full, blocks.part - G.proj_base.part};
             if (G.count) h->groups.push_back(G);
         }
-        h->proj_blocks = blocks;
         if ((e = cudaMalloc(&h->d_inst, sizeof(InstDesc))) != cudaSuccess ||
             (e = cudaMemcpy(h->d_inst, &h->inst_host, sizeof(InstDesc), cudaMemcpyHostToDevice)) != cudaSuccess ||
             (e = upload(&h->d_wfs, h->wfs_host)) != cudaSuccess) {
@@ -1479,10 +1452,8 @@ wfs_status wfs_measure_host(wfs_handle h, const float *screens_host, double t_s,
             pa.type == cudaMemoryTypeHost && pa.devicePointer != nullptr) {
             if (h->host_calls >= 2 && (e = cudaStreamWaitEvent(s, h->ev_done[i], 0)) != cudaSuccess)
                 return cuda_fail(h, e, "host-path wait");
-            h->screens_host_mapped = true;
             wfs_status st = measure_impl(h, static_cast<const float *>(pa.devicePointer), t_s, h->d_slopes_stage[i],
                                          nullptr, s);
-            h->screens_host_mapped = false;
             if (st != WFS_OK) return st;
             if ((e = cudaMemcpyAsync(slopes_host, h->d_slopes_stage[i], nsl * sizeof(float), cudaMemcpyDeviceToHost,
                                      s)) != cudaSuccess ||
@@ -1744,9 +1715,6 @@ wfs_status batch_fill(wfs_batch b, const float *const *screens, const double *t,
         d.noise = b->hs[i]->noise;
         b->hs[i]->last_stream = nullptr;
     }
-    bool aligned = true;
-    for (int i = 0; i < n; ++i) aligned = aligned && aligned16(screens[i]);
-    b->pa->stage_cap = (b->proj_stage > 0 && aligned) ? b->proj_stage : 0;
     for (size_t c = 0; c < b->classes.size(); ++c) {
         ShArgs &a = *b->sa[c];
         const BatchClass &bc = b->classes[c];
@@ -1765,7 +1733,6 @@ wfs_status batch_fill(wfs_batch b, const float *const *screens, const double *t,
 cudaError_t batch_build_graph(wfs_batch b) {
     cudaError_t e;
     if ((e = cudaGraphCreate(&b->graph, 0)) != cudaSuccess) return e;
-    b->graph_stage = b->pa->stage_cap;
     LaunchShape ps;
     project_launch_shape(*b->pa, b->proj_blocks, &ps);
     void *pargs[] = {(void *)b->pa};
@@ -1946,17 +1913,15 @@ wfs_status wfs_batch_create(int n, const wfs_handle *hs, wfs_batch *out) {
                 per[c].push_back(d);
             }
         }
-    int blocks = 0;
+    ProjRange blocks{0, 0};
     for (size_t c = 0; c < b->classes.size(); ++c) {
         BatchClass &bc = b->classes[c];
         bc.first = (int)b->wfs_host.size();
         for (WfsDesc d : per[c]) {
             d.subap_begin = bc.total;
             bc.total += d.n_valid;
-            d.proj_block_begin = blocks;
-            blocks += project_blocks(d);
-            if (project_box_floats(d) > b->proj_box) b->proj_box = project_box_floats(d);
-            merge_stage(b->proj_stage, bulk_stage_floats(d, hs[d.inst]->S));
+            place_blocks(d, blocks);
+            b->proj_rows = std::max(b->proj_rows, project_box_rows(d));
             b->wfs_host.push_back(d);
             ++bc.count;
         }
@@ -1985,9 +1950,9 @@ wfs_status wfs_batch_create(int n, const wfs_handle *hs, wfs_batch *out) {
     b->pa->wfs = b->d_wfs;
     b->pa->n_wfs = (int)b->wfs_host.size();
     b->pa->n_inst = n;
-    b->pa->box_cap = b->proj_box;
-    b->pa->stage_cap = b->proj_stage > 0 ? b->proj_stage : 0;
-    b->pa->n_blocks = b->proj_blocks;
+    b->pa->box_rows = b->proj_rows;
+    b->pa->n_full = b->proj_blocks.full;
+    b->pa->n_blocks = b->proj_blocks.full + b->proj_blocks.part;
     for (int i = 0; i < n; ++i) b->pa->max_layers = std::max(b->pa->max_layers, hs[i]->inst_host.n_layers);
     b->pa->work = b->d_work + 2 * b->classes.size() * (1 + kBatchSlots);
     b->pa->status = hs[0]->d_status;
@@ -2025,9 +1990,8 @@ wfs_status wfs_batch_measure(wfs_batch b, const float *const *screens, const dou
         if ((e = batch_launch_direct(b, s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
         return WFS_OK;
     }
-    // the projection node's kernel follows the screens' alignment, and a class has a noise node
-    // only while an instance of it has noise on: a change of either rebuilds the graph
-    bool same = b->graph_stage == b->pa->stage_cap;
+    // a class has a noise node only while an instance of it has noise on: a change rebuilds the graph
+    bool same = true;
     for (size_t c = 0; c < b->classes.size() && c < b->noise_nodes.size(); ++c)
         same = same && (b->classes[c].total <= 0 || (b->noise_nodes[c] != nullptr) == (b->sa[c]->split_noise != 0));
     if (b->exec && !same) batch_drop_graph(b);
@@ -2089,9 +2053,8 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
             d.t = t_s[pos[i]];
             d.noise = b->hs[i]->noise;
         }
-    int count = 0, blocks = 0, box = 0, stage = 0;
-    bool aligned = true;
-    for (int j = 0; j < n_active; ++j) aligned = aligned && aligned16(screens[j]);
+    int count = 0, rows = 0;
+    ProjRange blocks{0, 0};
     std::vector<int> cls_first(b->classes.size()), cls_count(b->classes.size()), cls_total(b->classes.size());
     for (size_t c = 0; c < b->classes.size(); ++c) {
         const BatchClass &bc = b->classes[c];
@@ -2103,10 +2066,8 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
             WfsDesc d = src;
             d.subap_begin = cls_total[c];
             cls_total[c] += d.n_valid;
-            d.proj_block_begin = blocks;
-            blocks += project_blocks(d);
-            if (project_box_floats(d) > box) box = project_box_floats(d);
-            merge_stage(stage, bulk_stage_floats(d, b->hs[src.inst]->S));
+            place_blocks(d, blocks);
+            rows = std::max(rows, project_box_rows(d));
             sl.h[count++] = d;
         }
         cls_count[c] = count - cls_first[c];
@@ -2118,15 +2079,14 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
     pa.inst = b->d_inst;
     pa.wfs = sl.d;
     pa.n_wfs = count;
-    pa.block_base = 0;
+    pa.block_base = pa.part_base = 0;
     pa.max_layers = 0;
     for (size_t i = 0; i < b->hs.size(); ++i) pa.max_layers = std::max(pa.max_layers, b->hs[i]->inst_host.n_layers);
     pa.work = b->d_work + 2 * b->classes.size() * (1 + kBatchSlots) + 2 * (1 + (size_t)slot);
     pa.n_inst = n;
-    pa.box_cap = box;
-    pa.stage_cap = (stage > 0 && aligned) ? stage : 0;
+    pa.box_rows = rows;
     pa.status = b->hs[0]->d_status;
-    if (blocks > 0 && (e = launch_project(pa, blocks, (cudaStream_t)stream)) != cudaSuccess)
+    if ((e = launch_project(pa, blocks, (cudaStream_t)stream)) != cudaSuccess)
         return cuda_fail(nullptr, e, "batch subset projection");
     for (size_t c = 0; c < b->classes.size(); ++c) {
         if (!cls_count[c] || !cls_total[c]) continue;
@@ -2445,9 +2405,8 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             pa.wfs = c.d_wfs;
             pa.n_wfs = ni;
             pa.n_inst = ni;
-            pa.box_cap = h->proj_box;
-            pa.stage_cap = h->proj_stage > 0 ? h->proj_stage : 0;
-            pa.block_base = 0;
+            pa.box_rows = h->proj_rows;
+            pa.block_base = pa.part_base = 0;
             pa.max_layers = 1;
             pa.work = c.work;
             pa.status = h->d_status;
@@ -2458,7 +2417,7 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
                 pa.dyn[i] = dyn;
             }
             sl = timed_begin(h, "project", s);
-            e = launch_project(pa, ni * c.blocks_per_wfs, s);
+            e = launch_project(pa, {ni * c.blocks_per_wfs.full, ni * c.blocks_per_wfs.part}, s);
             timed_end(h, sl, s);
             if (e != cudaSuccess) return cuda_fail(h, e, "calibration projection");
             memset(&sa, 0, offsetof(ShArgs, dyn));

@@ -31,7 +31,7 @@ constexpr int kMaxUniG = 40;         // 8 columns x 5 column pairs (n <= 10)
 
 struct InstDesc {                   // static per instance
     int n_layers, S;                // turbulent layers; mirror layers follow them (InstDyn::n_dm)
-    double ds;
+    double ds, inv_ds;              // screen pitch and 1 / ds
     double alt[kMaxProjLayers], vx[kMaxProjLayers], vy[kMaxProjLayers], x0[kMaxProjLayers],
         y0[kMaxProjLayers];
     uint64_t seed;
@@ -44,6 +44,12 @@ struct SliceDesc {
     int n;
     float w[kMaxNaSlices], k[kMaxNaSlices];
     float2 c[kMaxNaSlices][kMaxProjLayers];
+};
+
+// Projection blocks: of whole width (or of direct gathers), and narrower ones.  A launch hands out all
+// the whole ones first: the narrow ones fill its tail.
+struct ProjRange {
+    int full, part;
 };
 
 struct WfsDesc {                    // static per wavefront sensor
@@ -59,12 +65,13 @@ struct WfsDesc {                    // static per wavefront sensor
     const float *fill;              // [n_valid]
     const float2 *ktil;             // [n_valid][(2n-1)*n] elongation transfer (LGS only)
     long long opd_off, slope_off, int_off, det_off;  // into the instance's buffers (floats)
-    int proj_block_begin;           // first CTA of this WFS in the projection launch
+    // first whole-width and first narrow projection block of this WFS among its launch's (place_blocks)
+    int proj_block_begin, proj_part_begin;
     int subap_begin;                // first subaperture of this WFS in its spot launch
-    // projection by shared-memory tiles (pupil pitch <= screen pitch): runs of consecutive
-    // valid subapertures of one subaperture row, {sy, first valid index, count, sx of first}
+    // projection by screen boxes in shared memory (pupil pitch <= screen pitch): the blocks
+    // (build_segments)
     const int4 *segs;
-    int n_segs, tiled, seg_cols;    // seg_cols: largest run width in pupil columns
+    int n_segs, n_full, tiled;      // n_full: those of whole width, which come first
     // LGS uplink tip-tilt (null: off): the kernel k_uplink writes the spot's deflection times
     // the pupil pitch (OPD per pupil pixel, x and y) here before the projection adds it
     float2 *uplink;
@@ -92,15 +99,14 @@ struct ProjArgs {
     const InstDesc *inst;
     const WfsDesc *wfs;
     int n_wfs, n_inst;
-    int box_cap;                    // floats of shared memory for tables and screen box
-    int stage_cap;                  // floats of one screen box of the bulk-copy form (> 0: that
-                                    // form runs; 0: the cp.async form or direct gathers)
-    int block_base;                 // projection block of this launch's first block (a launch
-                                    // may cover a contiguous range of the WFS table)
-    int n_blocks;                   // blocks in this launch (set by the launcher)
+    int box_rows;                   // rows of the largest screen box of the launch (project_box_rows);
+                                    // 0: direct gathers only
+    // this launch's first blocks among the WFS table's (a launch may cover a contiguous range of it),
+    // its whole-width blocks and all of its blocks (the last two set by the launcher)
+    int block_base, part_base, n_full, n_blocks;
     int max_layers;                 // largest n_layers + n_dm of the launch's instances
     int *work;                      // ticket counter pair {next, CTAs done}, zero between
-                                    // launches, one launch at a time; null = one CTA per block
+                                    // launches, one launch at a time; null = a static split
     int *status;                    // device status word (limit errors)
     InstDyn dyn[kMaxInstances];
 };
@@ -241,22 +247,20 @@ struct LaunchShape {
 // Launchers (return the cudaGetLastError() of the launch).
 // after_uplink: the launch follows the uplink kernel on s as a programmatic dependent launch
 // (the projection waits for it before adding the uplink tilt).
-cudaError_t launch_project(const ProjArgs &a, int total_blocks, cudaStream_t s, bool after_uplink = false);
-cudaError_t project_launch_shape(const ProjArgs &a, int total_blocks, LaunchShape *out);
-// CTAs the projection needs for one WFS.
-int project_blocks(const WfsDesc &d);
-// Shared-memory floats the WFS's screen box needs (0 when it is projected by direct gathers).
-int project_box_floats(const WfsDesc &d);
-// Floats of one screen box of the bulk-copy projection for WFS d (0: not tiled).
-int project_stage_floats(const WfsDesc &d);
-// The bulk-copy projection's launch (tiled blocks through screen boxes moved by the bulk-copy
-// unit, direct-gather blocks as in k_project).
-cudaError_t project_bulk_launch_shape(const ProjArgs &a, int total_blocks, LaunchShape *out);
-// Runs of consecutive valid subapertures per subaperture row, at most max_count each.
-void build_segments(const std::vector<int32_t> &ids, int n_sub, int max_count, std::vector<int4> &segs,
-                    int *max_run);
-// Largest run (in subapertures) of one projection tile for n x n-pixel subapertures.
-int segment_max_count(int n);
+cudaError_t launch_project(const ProjArgs &a, ProjRange blocks, cudaStream_t s, bool after_uplink = false);
+cudaError_t project_launch_shape(const ProjArgs &a, ProjRange blocks, LaunchShape *out);
+// Blocks (warps' work) of one WFS in a projection launch.
+ProjRange project_blocks(const WfsDesc &d);
+// Gives WFS d the next blocks of a table that has r so far.
+void place_blocks(WfsDesc &d, ProjRange &r);
+// Screen rows of the WFS's boxes (0 when it is projected by direct gathers).
+int project_box_rows(const WfsDesc &d);
+// The blocks of a tiled WFS with n x n-pixel subapertures and the given valid ids, each up to 64 pupil
+// columns of a run of consecutive valid subapertures of one subaperture row by up to 11 of its pupil
+// rows: {subaperture row | first pupil row << 16, first valid index of the run, its first subaperture
+// column, first pupil column within the run | columns << 24}.  Returns how many have the whole width
+// (they come first).
+int build_segments(const std::vector<int32_t> &ids, int n_sub, int n, std::vector<int4> &segs);
 cudaError_t launch_ktil(const KtilArgs &a, cudaStream_t s);
 cudaError_t launch_noise(const float *E, int n, float ron, uint64_t seed, uint32_t wfs, double t,
                          uint32_t pixel0, float *C, cudaStream_t s);

@@ -1,12 +1,28 @@
-// k_project.cu -- layered frozen-flow projection (Sec. 4 "Open Loop generation": the layers'
-// screens are piled up, each shifted for the star's direction and for the temporal evolution;
-// for an LGS the pupil projection shrinks with altitude, c = 1 - h / range).  No Fresnel
-// propagation.  The coordinate arithmetic (FP64 per-layer offsets, FP32 per-pixel term with an
-// exact two-float split) is in proj_math.cuh; it keeps long runs (large v t) exact to FP64
-// rounding and the fractional coordinate accurate to ~1e-7 px.
+// k_project.cu -- the layered frozen-flow projection (Sec. 4 "Open Loop generation": each layer's
+// screen shifted for the star's direction and the wind, shrunk by the LGS cone c = 1 - h / range, and
+// the layers summed by bilinear interpolation).
 //
-// Output layout: per WFS, [n_valid][n][n] (subaperture-tiled), so the spot kernel reads each
-// subaperture's n*n OPD as one contiguous block.
+// A warp owns a block: up to 64 consecutive pupil columns of a run of subapertures by up to 11 pupil
+// rows of one subaperture row; lane i takes the columns i and i + 32.  Per layer, the box of screen
+// pixels that the block's taps touch (at most 68 x 12) is copied to the warp's own ring of three slots
+// by cp.async, two layers ahead of the interpolation; nothing but the warp itself waits for it, so the
+// warps of an SM run out of step and cover each other's copies.  The geometry of all of a block's
+// boxes is formed at its start, a layer per lane.  Going down a column, pupil row p + 1 falls on the
+// same screen row pair as row p or one row lower (the cone factor is at most one for a tiled WFS), so
+// a row's lower interpolated tap pair is the next row's upper pair; the two columns travel as packed
+// FP32x2 operations.
+//
+// A WFS whose pupil samples the screens more coarsely than one screen pixel, and every WFS of the
+// allocation-free entry point, is projected by direct gathers (proj_direct.cuh), 32 blocks of 2 x 2
+// pixels a warp.  Every form does the same per-tap arithmetic in the same order: the same OPD.
+//
+// Bound: issue and latency (45 % issue at 16 warps per SM), and at the start of a launch the instruction
+// fetches and the dependent loads of the first blocks: the rare copies are kept out of line for that
+// (with them inlined, 45 -> 49 us).  Measured against boxes of up to 400 columns moved by bulk copies of
+// two producer warps to eight consumer warps of a CTA (library events, L2 flushed): ELT frame 44.6 -> 42
+// us, 48 (LGS, slice) pairs of it 235 -> 209 us, 316 subapertures on one layer 15.0 -> 12.5 us, 64
+// measurements on one layer 96.5 -> 101 us; an uneven batch of 64 frames 477 -> 430 us.  Three slots,
+// 24 warps per SM, and preparing a block while the one before it runs gained nothing.
 #include <algorithm>
 #include <mutex>
 
@@ -16,327 +32,415 @@
 
 namespace gbwfs {
 
-constexpr int kProjThreads = 256;
+namespace {
 
-constexpr int kTilePixels = 4096;                         // pupil pixels per tiled CTA
-constexpr int kTilePx = kTilePixels / kProjThreads;       // per thread
+constexpr int kProjWarps = 8;
+constexpr int kProjThreads = 32 * kProjWarps;
+constexpr int kProjCtas = 2;                    // CTAs per SM
+constexpr int kBlockCols = 64;                  // pupil columns of a block
+constexpr int kBlockRows = 11;                  // most pupil rows of a block
+// A box has at most np + 1 rows and ncol + 4 columns (c <= 1: the taps' extent, the bilinear neighbour
+// and up to three columns for the 16-byte alignment); one more of each where c = 1 up to rounding.
+constexpr int kBoxCols = kBlockCols + 8;
+constexpr int kPitch = 4 * kBoxCols;            // bytes of a box row
+constexpr int kSlots = 2;
+constexpr int kRowPitch = kBlockRows + 1;       // row table of a layer
+constexpr int kOffsTable = 512;                 // (WFS, layer) offsets a CTA keeps for its whole launch
 
-__device__ __forceinline__ int wrap_index(int i, int S, bool pow2) {
-    if (pow2) return i & (S - 1);
-    int r = i % S;
+// The rows of a block: n pupil rows in equal parts of at most kBlockRows.
+__host__ __device__ inline int block_rows(int n) {
+    const int parts = (n + kBlockRows - 1) / kBlockRows;
+    return (n + parts - 1) / parts;
+}
+
+// One layer of a warp's block.
+struct __align__(16) LayerBox {
+    float c, cl, fu, fv;
+    const float *src;  // the box's first element in the screen
+    int bx0, by0;      // the box's first column and row, as offsets from the layer base
+    const float *scr;  // the layer
+    int cs, rs;        // the box's first screen column (a multiple of 4 but for kUnaligned) and row
+    int mode;          // kInside, kEdge, kUnaligned, or kNone
+    int cols, rows;    // its extent (kEdge, kUnaligned)
+    int pad;
+};
+// How a box is copied: by 16-byte words with the block's fixed extent; the same word by word across
+// the periodic screen's edges; element by element (rows without 16-byte alignment); not at all (the
+// taps do not fit, which does not happen: reported).
+enum { kInside = 0, kEdge = 1, kUnaligned = 2, kNone = 3 };
+
+// i in (-S, 2 S) wrapped into [0, S).
+__device__ __forceinline__ int wrap_once(int i, int S) {
+    i += i < 0 ? S : 0;
+    return i - (i >= S ? S : 0);
+}
+
+__device__ __forceinline__ int wrap_any(int i, int S) {
+    const int r = i % S;
     return r < 0 ? r + S : r;
 }
 
-constexpr int kOffsTable = 96;  // layer offsets a CTA keeps for every (WFS, layer) of its launch
-
-// One projection block (a tiled segment, or kProjThreads 2x2 pixel blocks); every thread of
-// the CTA calls it (its shared memory is free again once all threads have returned).  tab: the
-// CTA's layer offsets; with all_offs, entry w * max_layers + l for every WFS w of the launch
-// (filled once at the start of the kernel), else entries 0 .. L of the WFS last_wfs (refilled
-// when a block belongs to another WFS).
-__device__ __forceinline__ void project_one(const ProjArgs &a, const int bid, int &last_wfs, LayerOffs *tab,
-                                            bool all_offs) {
-
-    // the WFS owning this block: last entry whose first block is <= bid
-    int lo = 0, hi = a.n_wfs - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a.wfs[mid].proj_block_begin <= bid) lo = mid;
-        else hi = mid - 1;
-    }
-    const WfsDesc &W = a.wfs[lo];
-    const InstDesc &I = a.inst[W.inst];
-    const InstDyn &D = a.dyn[W.inst];
-    const int S = I.S;
-
-    const LayerOffs *s_off = all_offs ? tab + lo * a.max_layers : tab;
-    if (!all_offs && lo != last_wfs) {  // uniform: last_wfs was written before the caller's barrier
-        if ((int)threadIdx.x < proj_layers(I, D)) tab[threadIdx.x] = layer_offsets(I, W, D.t, threadIdx.x);
-        __syncthreads();
-        if (threadIdx.x == 0) last_wfs = lo;  // read again only after the caller's barrier
-    }
-
-    const bool pow2 = (S & (S - 1)) == 0;
-    if (W.tiled) {
-        // One run of consecutive subapertures of one subaperture row.  Each layer's screen
-        // footprint is staged in shared memory by cp.async; coordinates come from per-column
-        // and per-row tables (a pixel's screen column depends on its pupil column only).
-        // Tables and boxes are triple-buffered: in iteration l the CTA fills buffer
-        // (l + 1) mod 3, last read by layer l - 2, which every thread finished before the
-        // previous barrier; so one barrier per layer suffices (box l landed, tables l visible).
-        extern __shared__ float psm[];
-        __shared__ int4 s_geom[kMaxProjLayers];  // per layer: box origin (bx0, by0) and size (bw, bh)
-        const int4 sg = W.segs[bid - W.proj_block_begin];  // sy, v_first, count, sx0
-        const int n = W.n, nn = n * n, ncol = sg.z * n, L = proj_layers(I, D);
-        const int tab_floats = (6 * (ncol + n) + 3) & ~3;  // three tables, 16-byte aligned boxes
-        const int box_floats = ((a.box_cap - tab_floats) / 3) & ~3;
-        // buffer i: tables at tab0 + i (ncol + n), box at box0 + i box_floats
-        float2 *const tab0 = reinterpret_cast<float2 *>(psm);
-        float *const box0 = psm + tab_floats;
-        const float half = 0.5f * (float)(W.n_sub * n - 1);
-        // thread -> (pupil row p, columns ch + k nch, k < kTilePx): lanes of a warp take
-        // consecutive columns of one row, so their table and box reads fall in distinct banks
-        const int nch = (ncol + kTilePx - 1) / kTilePx, ntask = n * nch;  // ntask <= kProjThreads
-        const bool has_task = (int)threadIdx.x < ntask;
-        const int p = has_task ? (int)threadIdx.x / nch : 0, ch = (int)threadIdx.x - p * nch;
-        // acc[k / 2] holds the pixels k (x) and k + 1 (y), summed with packed FP32x2 operations
-        // (each half rounded as the scalar operation)
-        static_assert(kTilePx % 2 == 0, "pixels travel in pairs");
-        float2 acc[kTilePx / 2];
-#pragma unroll
-        for (int k = 0; k < kTilePx / 2; ++k) acc[k] = make_float2(0.0f, 0.0f);
-        // table entry j of layer l (column j < ncol, else row j - ncol): integer screen offset
-        // from the layer base (as float bits) and the fraction
-        auto coord = [&](int l, int j) -> float2 {
-            const bool col = j < ncol;
-            const float xr = col ? (float)(sg.w * n + j) - half : (float)(sg.x * n + (j - ncol)) - half;
-            int off;
-            float frac;
-            screen_offset(s_off[l].c, s_off[l].cl, col ? s_off[l].fu : s_off[l].fv, xr, off, frac);
-            return make_float2(__int_as_float(off), frac);
-        };
-        auto tables = [&](int l, float2 *t) {
-            for (int j = threadIdx.x; j < ncol + n; j += kProjThreads) t[j] = coord(l, j);
-        };
-        // Box origin (relative to the layer base) and size, the origin rounded down so that the
-        // box's first screen column is a multiple of 4: 16-byte copies when the layer's rows start
-        // on 16-byte boundaries (S % 4 == 0 and a 16-byte-aligned layer base), else 4-byte copies.
-        auto layer_vec = [&](int l) {
-            return (S & 3) == 0 && (reinterpret_cast<uintptr_t>(layer_screen(I, D, l)) & 15) == 0;
-        };
-        if ((int)threadIdx.x < L) {
-            const int l = threadIdx.x;
-            const bool vec = layer_vec(l);
-            int bx0 = __float_as_int(coord(l, 0).x), by0 = __float_as_int(coord(l, ncol).x);
-            int bw = __float_as_int(coord(l, ncol - 1).x) - bx0 + 2;
-            const int bh = __float_as_int(coord(l, ncol + n - 1).x) - by0 + 2;
-            if (vec) {
-                const int off = wrap_index(s_off[l].bu + bx0, S, pow2) & 3;
-                bx0 -= off;
-                bw = (bw + off + 3) & ~3;
-            }
-            s_geom[l] = make_int4(bx0, by0, bw, bh);
-        }
-        // returns false (for every thread) when the box would not fit
-        auto issue_box = [&](int l, float *box) -> bool {
-            const int4 gm = s_geom[l];
-            const int bx0 = gm.x, by0 = gm.y, bw = gm.z, bh = gm.w;
-            if (bw * bh > box_floats) return false;
-            const float *scr = layer_screen(I, D, l);
-            if (layer_vec(l)) {
-                // one warp per box row, one lane per 16-byte chunk
-                const int cw = bw >> 2, lane = threadIdx.x & 31, cbase = s_off[l].bu + bx0;
-                for (int r = threadIdx.x >> 5; r < bh; r += kProjThreads / 32) {
-                    const float *srow = scr + (size_t)wrap_index(s_off[l].bv + by0 + r, S, pow2) * S;
-                    float *drow = box + r * bw;
-                    for (int c4 = lane; c4 < cw; c4 += 32) {
-                        if (!guard(r * bw + 4 * c4 + 3 < box_floats, a.status)) continue;
-                        const float *src = srow + wrap_index(cbase + 4 * c4, S, pow2);
-                        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(drow + 4 * c4);
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-                    }
-                }
-            } else {
-                for (int r = 0; r < bh; ++r) {
-                    const float *grow = scr + (size_t)wrap_index(s_off[l].bv + by0 + r, S, pow2) * S;
-                    for (int c = threadIdx.x; c < bw; c += kProjThreads) {
-                        if (!guard(r * bw + c < box_floats, a.status)) continue;
-                        const float *src = grow + wrap_index(s_off[l].bu + bx0 + c, S, pow2);
-                        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(box + r * bw + c);
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-                    }
-                }
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            return true;
-        };
-        tables(0, tab0);
-        __syncthreads();  // geometry of every layer, tables of layer 0
-        bool fits = issue_box(0, box0);
-        for (int l = 0; l < L && fits; ++l) {
-            const int cur = l % 3, nxt = (l + 1) % 3;
-            const bool more = l + 1 < L;
-            bool fits_next = true;
-            if (more) {
-                tables(l + 1, tab0 + nxt * (ncol + n));
-                fits_next = issue_box(l + 1, box0 + nxt * box_floats);
-            }
-            if (more && fits_next)
-                asm volatile("cp.async.wait_group 1;" ::: "memory");
-            else
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncthreads();
-            const float2 *t = tab0 + cur * (ncol + n);
-            const float *box = box0 + cur * box_floats;
-            const int4 gm = s_geom[l];
-            const int bw = gm.z;
-            if (has_task) {
-                const float2 rp = t[ncol + p];
-                const float *brow = box + (__float_as_int(rp.x) - gm.y) * bw - gm.x;
-                const float2 gy = make_float2(rp.y, rp.y), m1 = make_float2(-1.0f, -1.0f);
-#pragma unroll
-                for (int k = 0; k < kTilePx; k += 2) {
-                    const int j = ch + k * nch, j2 = j + nch;
-                    if (j2 < ncol) {
-                        // two pixels: x - y as fma(y, -1, x) is the rounded difference
-                        const float2 ca = t[j], cb = t[j2];
-                        const float *b0 = brow + __float_as_int(ca.x), *b1 = brow + __float_as_int(cb.x);
-                        if (!guard(b0 >= box && b0 + bw + 1 < box + box_floats && b1 >= box &&
-                                       b1 + bw + 1 < box + box_floats,
-                                   a.status))
-                            continue;
-                        const float2 fx = make_float2(ca.y, cb.y);
-                        const float2 s00 = make_float2(b0[0], b1[0]), s01 = make_float2(b0[1], b1[1]);
-                        const float2 s10 = make_float2(b0[bw], b1[bw]), s11 = make_float2(b0[bw + 1], b1[bw + 1]);
-                        const float2 top = __ffma2_rn(fx, __ffma2_rn(s00, m1, s01), s00);
-                        const float2 bot = __ffma2_rn(fx, __ffma2_rn(s10, m1, s11), s10);
-                        acc[k / 2] = __fadd2_rn(acc[k / 2], __ffma2_rn(gy, __ffma2_rn(top, m1, bot), top));
-                    } else if (j < ncol) {
-                        const float2 cj = t[j];
-                        const float *b0 = brow + __float_as_int(cj.x);
-                        if (!guard(b0 >= box && b0 + bw + 1 < box + box_floats, a.status)) continue;
-                        const float s00 = b0[0], s01 = b0[1], s10 = b0[bw], s11 = b0[bw + 1];
-                        const float top = fmaf(cj.y, s01 - s00, s00);
-                        const float bot = fmaf(cj.y, s11 - s10, s10);
-                        acc[k / 2].x += fmaf(rp.y, bot - top, top);
-                    }
-                }
-            }
-            fits = fits_next;
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        if (!fits && threadIdx.x == 0 && a.status) atomicCAS(a.status, 0, 6 /* WFS_EUNSUPPORTED */);
-        if (has_task) {
-            // column j = v n + q of the segment -> subaperture v, column q; j advances by nch
-            float *opd = D.opd + W.opd_off + (size_t)sg.y * nn + p * n;
-            const int dv = nch / n, dq = nch - dv * n;
-            int v = ch / n, q = ch - v * n;
-            // the uplink tip-tilt as a plane over the pupil (zero when off); the uplink kernel may
-            // still be running (programmatic dependent launch): wait for it first
-            float2 up = make_float2(0.0f, 0.0f);
-            if (W.uplink) {
-                wait_prior_grid();
-                up = *W.uplink;
-            }
-            const float row_tilt = up.y * ((float)(sg.x * n + p) - half);
-#pragma unroll
-            for (int k = 0; k < kTilePx; ++k) {
-                const float xr = (float)(sg.w * n + ch + k * nch) - half;
-                if (ch + k * nch < ncol) opd[v * nn + q] = (k & 1 ? acc[k / 2].y : acc[k / 2].x) + fmaf(up.x, xr, row_tilt);
-                q += dq;
-                v += dv;
-                if (q >= n) {
-                    q -= n;
-                    ++v;
-                }
-            }
-        }
-        return;
-    }
-
-    project_direct<kProjThreads>(a, W, I, D, s_off, bid, threadIdx.x);
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy4(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 
-// Blocks 0 .. n_blocks of this launch.  Each CTA starts with block blockIdx.x; with a.work the
-// grid holds only as many CTAs as fit at once and each draws its next block from the ticket
+// Shared memory of a CTA (bytes): per warp kSlots boxes of box_rows rows, the row tables and the
+// geometry of the layers' boxes; then the launch's layer offsets, when they fit.
+struct ProjSmem {
+    int box, rows, geo, warp, tab, total;
+};
+__host__ __device__ inline ProjSmem proj_smem(int box_rows, int max_layers, int n_wfs) {
+    ProjSmem s;
+    s.box = box_rows * kPitch;
+    s.rows = kSlots * s.box;
+    s.geo = s.rows + max_layers * kRowPitch * (int)sizeof(float2);
+    s.warp = box_rows > 0 ? s.geo + max_layers * (int)sizeof(LayerBox) : 0;
+    s.tab = kProjWarps * s.warp;
+    const int entries = n_wfs * max_layers <= kOffsTable ? n_wfs * max_layers : kProjWarps * max_layers;
+    s.total = s.tab + ((entries * (int)sizeof(LayerOffs) + 15) & ~15);
+    return s;
+}
+
+// Bilinear taps of two columns (a, b) on the box row at byte offset off, interpolated across with the
+// columns' fractions (x - y as fma(y, -1, x): the rounded difference).
+__device__ __forceinline__ float2 lerp_at(const char *pa, const char *pb, int off, float2 fx) {
+    const float *ra = reinterpret_cast<const float *>(pa + off), *rb = reinterpret_cast<const float *>(pb + off);
+    const float2 s0 = make_float2(ra[0], rb[0]), s1 = make_float2(ra[1], rb[1]);
+    return __ffma2_rn(fx, __ffma2_rn(s0, make_float2(-1.0f, -1.0f), s1), s0);
+}
+
+// R pupil rows whose box rows step by 0 or 1: straight-line code, so that the taps of later rows load
+// while earlier rows are interpolated.  A step of 0 keeps the row pair (its lower pair is recomputed
+// from the same taps: the same value).  rows[i]: byte offset of the lower box row (int bits), fraction.
+template <int R>
+__device__ __forceinline__ void rows_unit(float2 (&acc)[kBlockRows], const float2 *rows, const char *pa, const char *pb,
+                                          float2 fx) {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    float2 rp[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) rp[i] = rows[i];
+    int prev = __float_as_int(rp[0].x);
+    float2 top = lerp_at(pa, pb, prev - kPitch, fx);
+    float2 bot = lerp_at(pa, pb, prev, fx);
+    acc[0] = __fadd2_rn(acc[0], __ffma2_rn(make_float2(rp[0].y, rp[0].y), __ffma2_rn(top, m1, bot), top));
+#pragma unroll
+    for (int i = 1; i < R; ++i) {
+        const int off = __float_as_int(rp[i].x);
+        const float2 nb = lerp_at(pa, pb, off, fx);
+        const bool same = off == prev;
+        top = make_float2(same ? top.x : bot.x, same ? top.y : bot.y);
+        bot = nb;
+        prev = off;
+        acc[i] = __fadd2_rn(acc[i], __ffma2_rn(make_float2(rp[i].y, rp[i].y), __ffma2_rn(top, m1, bot), top));
+    }
+}
+
+// The copy of a box across the periodic screen's edges (word by word) or of rows without 16-byte
+// alignment (element by element).  Out of line: few boxes take it, and the kernel's code stays short.
+__device__ __noinline__ void copy_box_slow(const LayerBox *b, uint32_t dst, int S, int lane) {
+    const float *scr = b->scr;
+    const int cs = b->cs, rs = b->rs;
+    if (b->mode == kEdge) {
+        const int w4 = b->cols >> 2, n_words = b->rows * w4;
+        for (int idx = lane; idx < n_words; idx += 32) {
+            const int r = idx / w4, w = idx - r * w4;
+            copy16(dst + r * kPitch + 16 * w, scr + (size_t)wrap_any(rs + r, S) * S + wrap_any(cs + 4 * w, S));
+        }
+    } else {
+        const int w = b->cols, n_el = b->rows * w;
+        for (int idx = lane; idx < n_el; idx += 32) {
+            const int r = idx / w, c = idx - r * w;
+            copy4(dst + r * kPitch + 4 * c, scr + (size_t)wrap_any(rs + r, S) * S + wrap_any(cs + c, S));
+        }
+    }
+}
+
+// A warp's block seg (of W.segs) of a tiled WFS.
+__device__ __forceinline__ void project_block(const ProjArgs &a, const ProjSmem &L, const WfsDesc &W, const InstDesc &I,
+                                              const InstDyn &D, const LayerOffs *wt, int seg, char *scratch, int lane) {
+    const int4 sg = __ldg(W.segs + seg);
+    // sg: subaperture row | first pupil row << 16, first valid index and column of the run,
+    // first pupil column of the block within the run | columns << 24
+    const int n = W.n, sy = sg.x & 0xFFFF, p0 = sg.x >> 16, col0 = sg.w & 0xFFFFFF, ncol = sg.w >> 24;
+    const int np = min(block_rows(n), n - p0);
+    const int S = I.S, layers = proj_layers(I, D), n_scr = I.n_layers;
+    const float half = 0.5f * (float)(W.n_sub * n - 1);
+    const float x_first = (float)(sg.z * n + col0) - half, y_first = (float)(sy * n + p0) - half;
+    LayerBox *geo = reinterpret_cast<LayerBox *>(scratch + L.geo);
+    // 16-byte words and rows of a box copied by words
+    const int words = (ncol + 7) >> 2, box_rows = np + 1;
+    bool unit = true;  // every layer's box rows step by 0 or 1 from one pupil row to the next
+    for (int l = lane; l < layers; l += 32) {
+        const LayerOffs o = wt[l];
+        LayerBox b;
+        b.scr = l < n_scr ? D.screens + (size_t)l * S * S : D.dm + (size_t)(l - n_scr) * S * S;
+        b.c = o.c;
+        b.cl = o.cl;
+        b.fu = o.fu;
+        b.fv = o.fv;
+        int c0, c1, r0, r1;
+        float f, f0;
+        screen_offset(o.c, o.cl, o.fu, x_first, c0, f);
+        screen_offset(o.c, o.cl, o.fu, x_first + (float)(ncol - 1), c1, f);
+        screen_offset(o.c, o.cl, o.fv, y_first, r0, f0);
+        screen_offset(o.c, o.cl, o.fv, y_first + (float)(np - 1), r1, f);
+        // a step of 2 needs c = 1 up to rounding and a row on a screen row up to rounding
+        unit = unit && (o.c < 0.999999f || (f0 > 1e-4f && f0 < 0.9999f));
+        const bool vec = (S & 3) == 0 && (reinterpret_cast<uintptr_t>(b.scr) & 15) == 0;
+        // |c x / ds| < S (checked at creation), and the base is in [0, S)
+        const int cs = wrap_once(o.bu + c0, S), al = vec ? cs & 3 : 0;
+        b.cs = cs - al;
+        b.rs = wrap_once(o.bv + r0, S);
+        b.src = b.scr + (size_t)b.rs * S + b.cs;
+        b.bx0 = c0 - al;
+        b.by0 = r0;
+        b.cols = (c1 - c0 + 2 + al + 3) & ~3;
+        b.rows = r1 - r0 + 2;
+        const bool fits = c1 >= c0 && r1 >= r0 && b.cols <= kBoxCols && b.rows * kPitch <= L.box;
+        b.mode = !fits ? kNone
+                 : !vec ? kUnaligned
+                 : b.cs + 4 * words <= S && b.rs + box_rows <= S && b.cols <= 4 * words && b.rows <= box_rows ? kInside
+                                                                                                        : kEdge;
+        if (!fits && a.status) atomicCAS(a.status, 0, 6 /* WFS_EUNSUPPORTED */);
+        geo[l] = b;
+    }
+    unit = __all_sync(0xffffffffu, unit);
+    __syncwarp();
+
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(scratch);
+    // half a warp per box row: word lane mod 16 of rows half + 2 i; then the rows' last words, a row
+    // per lane (and half)
+    const int word = lane & 15, hrow = lane >> 4;
+    const bool word_on = word < words, tail_on = words > 16 && lane < box_rows;
+    auto copy_box = [&](int l, int slot) {
+        const LayerBox &b = geo[l];
+        const uint32_t dst = ring + (uint32_t)(slot * L.box);
+        const int mode = b.mode;
+        if (mode == kInside) {
+            const float *src = b.src;
+            const float *sw = src + hrow * S + 4 * word;
+            const uint32_t dw = dst + hrow * kPitch + 16 * word;
+#pragma unroll
+            for (int i = 0; i < (kBlockRows + 2) / 2; ++i)
+                if (word_on && 2 * i + hrow < box_rows) copy16(dw + 2 * i * kPitch, sw + (size_t)(2 * i) * S);
+            if (tail_on) copy16(dst + lane * kPitch + 256, src + (size_t)lane * S + 64);
+        } else if (mode != kNone) {
+            copy_box_slow(&b, dst, S, lane);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    const float xa = x_first + (float)lane, xb = xa + 32.0f;
+    float2 acc[kBlockRows];
+#pragma unroll
+    for (int i = 0; i < kBlockRows; ++i) acc[i] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int l = 0; l < kSlots - 1; ++l) {
+        if (l < layers) copy_box(l, l);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // every layer's row table while the first boxes travel, a (layer, row) per lane: byte offset of the
+    // lower box row, fraction
+    float2 *rows = reinterpret_cast<float2 *>(scratch + L.rows);
+    {
+        const int per = 32 / np, l0 = lane / np, p = lane - l0 * np;
+        const float y = y_first + (float)p;
+        for (int l = l0; l < layers && l0 < per; l += per) {
+            const LayerBox &b = geo[l];
+            int off;
+            float fr;
+            screen_offset(b.c, b.cl, b.fv, y, off, fr);
+            const int br = min(max(off - b.by0, 0), b.rows - 2);
+            rows[l * kRowPitch + p] = make_float2(__int_as_float((br + 1) * kPitch), fr);
+        }
+    }
+    int slot = 0;
+    for (int l = 0; l < layers; ++l) {
+        // the slot of layer l + kSlots - 1 was read for the layer before l (a warp barrier ago)
+        const int ahead = slot == 0 ? kSlots - 1 : slot - 1;
+        if (l + kSlots - 1 < layers) copy_box(l + kSlots - 1, ahead);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        const LayerBox &b = geo[l];
+        int oa, ob;
+        float2 fx;
+        screen_offset(b.c, b.cl, b.fu, xa, oa, fx.x);
+        screen_offset(b.c, b.cl, b.fu, xb, ob, fx.y);
+        guard(lane >= ncol || (oa - b.bx0 >= 0 && oa - b.bx0 + 1 < b.cols), a.status);
+        // columns kept inside the box (those past the block's are computed and dropped)
+        const int ca = min(max(oa - b.bx0, 0), kBoxCols - 2), cb = min(max(ob - b.bx0, 0), kBoxCols - 2);
+        const bool fits = b.mode != kNone;
+        const char *box = scratch + slot * L.box;
+        const char *pa = box + 4 * ca, *pb = box + 4 * cb;
+        const float2 *rt = rows + l * kRowPitch;
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
+        __syncwarp();  // every lane's copies of layer l, and the row tables
+        if (fits && unit) {
+            switch (np) {
+#define GBWFS_ROWS_CASE(R) \
+    case R: rows_unit<R>(acc, rt, pa, pb, fx); break;
+                GBWFS_ROWS_CASE(1) GBWFS_ROWS_CASE(2) GBWFS_ROWS_CASE(3) GBWFS_ROWS_CASE(4)
+                GBWFS_ROWS_CASE(5) GBWFS_ROWS_CASE(6) GBWFS_ROWS_CASE(7) GBWFS_ROWS_CASE(8)
+                GBWFS_ROWS_CASE(9) GBWFS_ROWS_CASE(10) GBWFS_ROWS_CASE(11)
+#undef GBWFS_ROWS_CASE
+                default: break;
+            }
+        } else if (fits) {
+            const float2 m1 = make_float2(-1.0f, -1.0f);
+#pragma unroll
+            for (int i = 0; i < kBlockRows; ++i)
+                if (i < np) {
+                    const float2 rp = rt[i];
+                    const int o = __float_as_int(rp.x);
+                    const float2 top = lerp_at(pa, pb, o - kPitch, fx), bot = lerp_at(pa, pb, o, fx);
+                    acc[i] = __fadd2_rn(acc[i], __ffma2_rn(make_float2(rp.y, rp.y), __ffma2_rn(top, m1, bot), top));
+                }
+        }
+        __syncwarp();  // the slot may be refilled
+        slot = slot == kSlots - 1 ? 0 : slot + 1;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+
+    // the uplink tip-tilt as a plane over the pupil (zero when off); the uplink kernel may still be
+    // running (programmatic dependent launch): wait for it first
+    float2 up = make_float2(0.0f, 0.0f);
+    if (W.uplink) {
+        wait_prior_grid();
+        up = *W.uplink;
+    }
+    float *opd = D.opd + W.opd_off + (size_t)sg.y * n * n;
+    const int ta = col0 + lane, tb = ta + 32, va = ta / n, vb = tb / n;
+    float *da = opd + (size_t)va * n * n + (ta - va * n), *db = opd + (size_t)vb * n * n + (tb - vb * n);
+    const bool on_a = lane < ncol, on_b = lane + 32 < ncol;
+    da += p0 * n;
+    db += p0 * n;
+    const bool tilt = W.uplink != nullptr;
+#pragma unroll
+    for (int i = 0; i < kBlockRows; ++i)
+        if (i < np) {
+            if (tilt) {
+                const float y = y_first + (float)i;
+                acc[i].x += fmaf(up.x, xa, up.y * y);
+                acc[i].y += fmaf(up.x, xb, up.y * y);
+            }
+            if (on_a) da[i * n] = acc[i].x;
+            if (on_b) db[i * n] = acc[i].y;
+        }
+}
+
+}  // namespace
+
+// Blocks 0 .. n_blocks of this launch.  Each warp starts with a block of its own; with a.work the
+// grid holds only as many CTAs as fit at once and each warp draws its next block from the ticket
 // counter (issued at the top, consumed after the block), so CTAs that start late take fewer
 // blocks and no partial last wave is left; the last CTA to finish resets the counter.
-__global__ void __launch_bounds__(kProjThreads, 3) k_project(const __grid_constant__ ProjArgs a) {
+__global__ void __launch_bounds__(kProjThreads, kProjCtas) k_project(const __grid_constant__ ProjArgs a) {
     allow_dependent_grid();  // every CTA of this grid is resident or done: the spot kernel may start
-    __shared__ int s_next, s_last_wfs;
-    __shared__ LayerOffs s_tab[kOffsTable];
-    // the layer offsets of every (WFS, layer) of this launch, once per CTA, when they fit
+    extern __shared__ __align__(16) char psm[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const ProjSmem L = proj_smem(a.box_rows, a.max_layers, a.n_wfs);
+    LayerOffs *tab = reinterpret_cast<LayerOffs *>(psm + L.tab);
+    // the layer offsets of every (WFS, layer) of this launch, once per CTA, when they fit; else a
+    // warp forms those of its block's WFS
     const bool all_offs = a.n_wfs * a.max_layers <= kOffsTable;
     if (all_offs) {
         for (int i = threadIdx.x; i < a.n_wfs * a.max_layers; i += blockDim.x) {
             const int w = i / a.max_layers, l = i - w * a.max_layers;
             const WfsDesc &W = a.wfs[w];
             const InstDesc &I = a.inst[W.inst];
-            if (l < proj_layers(I, a.dyn[W.inst])) s_tab[i] = layer_offsets(I, W, a.dyn[W.inst].t, l);
+            if (l < proj_layers(I, a.dyn[W.inst])) tab[i] = layer_offsets(I, W, a.dyn[W.inst].t, l);
         }
+        __syncthreads();
     }
-    if (threadIdx.x == 0) s_last_wfs = -1;
-    __syncthreads();
-    int blk = blockIdx.x;
-    while (blk < a.n_blocks) {
+    char *scratch = psm + wib * L.warp;
+    const int nwarps = gridDim.x * kProjWarps;
+    int last = -1;
+    // consecutive blocks go to different CTAs, so that a launch of few blocks reaches every SM
+    for (int blk = wib * gridDim.x + blockIdx.x; blk < a.n_blocks;) {
         int ticket = 0;
-        if (a.work && threadIdx.x == 0) ticket = atomicAdd(a.work, 1);
-        project_one(a, blk + a.block_base, s_last_wfs, s_tab, all_offs);
-        __syncthreads();  // the block's shared memory is free; orders s_next
-        if (a.work) {
-            if (threadIdx.x == 0) s_next = (int)gridDim.x + ticket;
-            __syncthreads();
-            blk = s_next;
-        } else {
-            blk += gridDim.x;
+        if (a.work && lane == 0) ticket = atomicAdd(a.work, 1);
+        // the WFS owning this block: last entry whose first block of the kind is <= bid
+        const bool part = blk >= a.n_full;
+        const int bid = part ? blk - a.n_full + a.part_base : blk + a.block_base;
+        int lo = 0, hi = a.n_wfs - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(part ? &a.wfs[mid].proj_part_begin : &a.wfs[mid].proj_block_begin) <= bid) lo = mid;
+            else hi = mid - 1;
         }
-    }
-    if (a.work && threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(a.work + 1, 1) == (int)gridDim.x - 1) {
-            a.work[0] = 0;
-            a.work[1] = 0;
+        const WfsDesc &W = a.wfs[lo];
+        const InstDesc &I = a.inst[W.inst];
+        const InstDyn &D = a.dyn[W.inst];
+        const LayerOffs *wt = all_offs ? tab + lo * a.max_layers : tab + wib * a.max_layers;
+        if (!all_offs && lo != last) {
+            __syncwarp();  // earlier reads of the warp's offsets are done
+            for (int l = lane; l < proj_layers(I, D); l += 32) tab[wib * a.max_layers + l] = layer_offsets(I, W, D.t, l);
+            last = lo;
+            __syncwarp();
         }
+        const int seg = part ? W.n_full + bid - W.proj_part_begin : bid - W.proj_block_begin;
+        if (W.tiled && a.box_rows > 0) project_block(a, L, W, I, D, wt, seg, scratch, lane);
+        else project_direct<32>(a, W, I, D, wt, seg, lane);
+        __syncwarp();
+        blk = a.work ? nwarps + __shfl_sync(0xffffffffu, ticket, 0) : blk + nwarps;
     }
-}
-
-int segment_max_count(int n) {
-    // a segment of c subaperture columns spans c n pupil columns: at most two per consumer thread
-    // of the bulk-copy projection (256 threads; row groups of whole warps over half the columns,
-    // at most 16 rows per thread), and n rows x ceil(c n / kTilePx) column sets <= kProjThreads
-    // for the cp.async form, which takes the same segments
-    auto ok = [&](int c) {
-        const int ncol = c * n, Tg = ((ncol + 1) / 2 + 31) & ~31;
-        if (Tg > 256) return false;
-        const int G = std::min(n, 256 / Tg), RG = (n + G - 1) / G;
-        return RG <= 16 && n * ((ncol + kTilePx - 1) / kTilePx) <= kProjThreads;
-    };
-    int c = 1;
-    while (ok(c + 1)) ++c;
-    return c;
-}
-
-int project_blocks(const WfsDesc &d) {
-    if (d.tiled) return d.n_segs;
-    const int nb = (d.n + 1) / 2;
-    return (d.n_valid * nb * nb + kProjThreads - 1) / kProjThreads;
-}
-
-int project_box_floats(const WfsDesc &d) {
-    if (!d.tiled) return 0;
-    // three sets of coordinate tables (3 x (ncol + n) float2) and three boxes of at most
-    // (ncol + 2) x (n + 2) screen pixels (padded for the 16-byte alignment)
-    return 6 * (d.seg_cols + d.n) + 4 + 3 * ((d.seg_cols + 9) * (d.n + 3) + 4);
-}
-
-void build_segments(const std::vector<int32_t> &ids, int n_sub, int max_count, std::vector<int4> &segs,
-                    int *max_run) {
-    segs.clear();
-    *max_run = 0;
-    for (size_t v = 0; v < ids.size(); ++v) {
-        const int sy = ids[v] / n_sub, sx = ids[v] - sy * n_sub;
-        if (!segs.empty()) {
-            int4 &b = segs.back();
-            if (b.x == sy && b.w + b.z == sx && b.z < max_count) {
-                ++b.z;
-                if (b.z > *max_run) *max_run = b.z;
-                continue;
+    if (a.work) {
+        __syncthreads();  // every warp of the CTA has drawn past the end
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicAdd(a.work + 1, 1) == (int)gridDim.x - 1) {
+                a.work[0] = 0;
+                a.work[1] = 0;
             }
         }
-        segs.push_back(make_int4(sy, (int)v, 1, sx));
-        if (*max_run < 1) *max_run = 1;
     }
-    // longest runs first: with the projection's ticket order the short ones fill the tail
-    std::stable_sort(segs.begin(), segs.end(), [](const int4 &x, const int4 &y) { return x.z > y.z; });
 }
 
-cudaError_t launch_project(const ProjArgs &a, int total_blocks, cudaStream_t s, bool after_uplink) {
-    if (total_blocks <= 0) return cudaSuccess;
+ProjRange project_blocks(const WfsDesc &d) {
+    if (d.tiled) return {d.n_full, d.n_segs - d.n_full};
+    const int nb = (d.n + 1) / 2;
+    return {(d.n_valid * nb * nb + 31) / 32, 0};
+}
+
+void place_blocks(WfsDesc &d, ProjRange &r) {
+    const ProjRange n = project_blocks(d);
+    d.proj_block_begin = r.full;
+    d.proj_part_begin = r.part;
+    r.full += n.full;
+    r.part += n.part;
+}
+
+int project_box_rows(const WfsDesc &d) { return d.tiled ? block_rows(d.n) + 2 : 0; }
+
+int build_segments(const std::vector<int32_t> &ids, int n_sub, int n, std::vector<int4> &segs) {
+    segs.clear();
+    const int R = block_rows(n);
+    for (size_t v = 0; v < ids.size();) {
+        const int sy = ids[v] / n_sub, sx = ids[v] - sy * n_sub;
+        size_t e = v + 1;  // the run of consecutive valid subapertures of this row
+        while (e < ids.size() && ids[e] == ids[e - 1] + 1 && ids[e] / n_sub == sy) ++e;
+        const int cols = (int)(e - v) * n;
+        for (int c = 0; c < cols; c += kBlockCols)
+            for (int p = 0; p < n; p += R)
+                segs.push_back(make_int4(sy | p << 16, (int)v, sx, c | std::min(kBlockCols, cols - c) << 24));
+        v = e;
+    }
+    std::stable_sort(segs.begin(), segs.end(), [](const int4 &x, const int4 &y) { return x.w >> 24 > y.w >> 24; });
+    int full = 0;
+    while (full < (int)segs.size() && segs[full].w >> 24 == kBlockCols) ++full;
+    return full;
+}
+
+cudaError_t launch_project(const ProjArgs &a, ProjRange blocks, cudaStream_t s, bool after_uplink) {
+    if (blocks.full + blocks.part <= 0) return cudaSuccess;
     LaunchShape sh;
-    cudaError_t e = project_launch_shape(a, total_blocks, &sh);
+    cudaError_t e = project_launch_shape(a, blocks, &sh);
     if (e != cudaSuccess) return e;
     ProjArgs b = a;
-    b.n_blocks = total_blocks;
+    b.n_full = blocks.full;
+    b.n_blocks = blocks.full + blocks.part;
     void *args[] = {(void *)&b};
     if (!after_uplink) return cudaLaunchKernel(sh.func, sh.grid, sh.block, args, sh.smem, s);
     cudaLaunchConfig_t cfg = {};
@@ -352,43 +456,29 @@ cudaError_t launch_project(const ProjArgs &a, int total_blocks, cudaStream_t s, 
     return cudaLaunchKernelExC(&cfg, sh.func, args);
 }
 
-cudaError_t project_launch_shape(const ProjArgs &a, int total_blocks, LaunchShape *out) {
-    // screen boxes moved by the bulk-copy unit where the launch's screens allow it
-    if (a.stage_cap > 0) return project_bulk_launch_shape(a, total_blocks, out);
-    const size_t smem = (size_t)a.box_cap * sizeof(float) + (a.box_cap ? 64 : 0);
-    // the kernel's dynamic shared-memory limit is process-wide: only ever raise it, so that a
-    // smaller request (the direct-gather launches ask for none) cannot lower it between another
-    // thread's setting and its launch
-    cudaError_t e = cudaSuccess;
+cudaError_t project_launch_shape(const ProjArgs &a, ProjRange blocks, LaunchShape *out) {
+    const int total_blocks = blocks.full + blocks.part;
+    const int smem = proj_smem(a.box_rows, a.max_layers, a.n_wfs).total;
+    // the dynamic shared-memory limit is process-wide: set once per device, to the most a CTA may have
+    static std::mutex m;
+    static bool set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
     {
-        static std::mutex m;
-        static size_t raised[64] = {};  // per device ordinal
-        int d = 0;
-        if ((e = cudaGetDevice(&d)) != cudaSuccess) return e;
         std::lock_guard<std::mutex> lk(m);
-        if (d < 0 || d >= 64 || smem > raised[d]) {
-            if ((e = cudaFuncSetAttribute(k_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        if (dev < 0 || dev >= 64 || !set[dev]) {
+            if ((e = cudaFuncSetAttribute(k_project, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) != cudaSuccess)
                 return e;
-            if (d >= 0 && d < 64) raised[d] = smem;
+            if (dev >= 0 && dev < 64) set[dev] = true;
         }
     }
-    int grid = total_blocks > 0 ? total_blocks : 1;
+    int grid = std::max(1, (total_blocks + kProjWarps - 1) / kProjWarps);
+    if (total_blocks < 152 * kProjWarps) grid = std::min(std::max(total_blocks, 1), 152);  // every SM
     if (a.work) {
-        // resident capacity for this shared-memory size (cached per thread)
-        static thread_local size_t c_smem = (size_t)-1;
-        static thread_local int c_dev = -1, c_cap = 0;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (smem != c_smem || dev != c_dev) {
-            int per_sm = 0, sms = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_project, kProjThreads, smem)) != cudaSuccess ||
-                (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-                return e;
-            c_smem = smem;
-            c_dev = dev;
-            c_cap = per_sm * sms;
-        }
-        if (c_cap > 0 && grid > c_cap) grid = c_cap;
+        // resident CTAs: two per SM where shared memory allows
+        const int per_sm = std::max(1, std::min(kProjCtas, 227 * 1024 / (smem + 1024)));
+        grid = std::min(grid, 152 * per_sm);
     }
     out->func = (const void *)k_project;
     out->grid = dim3(grid);

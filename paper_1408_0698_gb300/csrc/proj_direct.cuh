@@ -11,7 +11,7 @@
 
 namespace gbwfs {
 
-// Block bid (kThreads 2x2 blocks) of WFS W; s_off: the WFS's layer offsets; tid < kThreads.
+// Block bid (kThreads 2x2 blocks) of WFS W, counted within W; s_off: the WFS's layer offsets; tid < kThreads.
 template <int kThreads>
 __device__ __forceinline__ void project_direct(const ProjArgs &a, const WfsDesc &W, const InstDesc &I,
                                                const InstDyn &D, const LayerOffs *s_off, int bid, int tid) {
@@ -19,7 +19,7 @@ __device__ __forceinline__ void project_direct(const ProjArgs &a, const WfsDesc 
     const bool pow2 = (S & (S - 1)) == 0;
     // each thread: one 2x2 block of pupil pixels (rows p, p+1; columns q, q+1) of one subaperture
     const int n = W.n, nn = n * n, nb = (n + 1) >> 1, nbb = nb * nb;
-    const int blk = (bid - W.proj_block_begin) * kThreads + tid;
+    const int blk = bid * kThreads + tid;
     if (blk >= W.n_valid * nbb) return;
     const int v = blk / nbb, r = blk - v * nbb, bp = r / nb, bq = r - bp * nb;
     if (!guard(v < W.n_valid, a.status)) return;

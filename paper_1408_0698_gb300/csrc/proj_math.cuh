@@ -37,15 +37,22 @@ __device__ __forceinline__ LayerOffs layer_offsets(const InstDesc &I, const WfsD
     const int S = I.S;
     const double h = I.alt[l];
     const double c = W.is_lgs ? 1.0 - h / W.range_m : 1.0;
-    const double inv_ds = 1.0 / I.ds;
+    const double inv_ds = I.inv_ds;
     const double ou = 0.5 * S + (W.theta_x * h - (I.x0[l] + I.vx[l] * t)) * inv_ds;
     const double ov = 0.5 * S + (W.theta_y * h - (I.y0[l] + I.vy[l] * t)) * inv_ds;
     const double bu = floor(ou), bv = floor(ov);
     LayerOffs o;
     o.fu = (float)(ou - bu);
     o.fv = (float)(ov - bv);
-    // base index mod S (exact: bu, bv are integers well inside 2^53)
-    long long iu = (long long)bu % S, iv = (long long)bv % S;
+    // base index mod S (exact: bu, bv are integers well inside 2^53; 32-bit division where they fit)
+    long long iu, iv;
+    if (fabs(bu) < 2147483647.0 && fabs(bv) < 2147483647.0) {
+        iu = (int)bu % S;
+        iv = (int)bv % S;
+    } else {
+        iu = (long long)bu % S;
+        iv = (long long)bv % S;
+    }
     if (iu < 0) iu += S;
     if (iv < 0) iv += S;
     o.bu = (int)iu;

@@ -216,6 +216,7 @@ extern "C" wfs_status wfs_measure_one_static(const wfs_telescope *tel, const wfs
     h_inst.n_layers = L->n_layers;
     h_inst.S = L->screen_size;
     h_inst.ds = L->screen_dx_m;
+    h_inst.inv_ds = 1.0 / h_inst.ds;
     for (int l = 0; l < L->n_layers; ++l) {
         h_inst.alt[l] = L->alt_m[l];
         h_inst.vx[l] = L->wind_vx_mps[l];
@@ -261,10 +262,9 @@ extern "C" wfs_status wfs_measure_one_static(const wfs_telescope *tel, const wfs
     h_pa.wfs = d_wfs;
     h_pa.n_wfs = 1;
     h_pa.n_inst = 1;
-    h_pa.box_cap = 0;  // direct gathers: no projection tiles in the static scratch
-    h_pa.stage_cap = 0;
-    h_pa.block_base = 0;
-    h_pa.work = nullptr;  // one CTA per block
+    h_pa.box_rows = 0;  // direct gathers: no block tables in the static scratch
+    h_pa.block_base = h_pa.part_base = 0;
+    h_pa.work = nullptr;
     h_pa.max_layers = h_inst.n_layers;
     h_pa.status = (int *)(base + o_status);
     h_pa.dyn[0] = dyn;
