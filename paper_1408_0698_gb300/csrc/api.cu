@@ -869,7 +869,7 @@ wfs_status calib_prepare(wfs_loop lp, int gs) {
     if ((e = cudaMalloc(&c.d_wfs, sizeof(WfsDesc) * kMaxInstances)) != cudaSuccess) return bail(e, "calibration table");
     if ((e = cudaMalloc(&c.d_inst, sizeof(InstDesc) * in.size())) != cudaSuccess) return bail(e, "calibration table");
     if ((e = cudaMalloc(&c.opd, sizeof(float) * c.opd_stride * kMaxInstances)) != cudaSuccess ||
-        (e = cudaMalloc(&c.slopes, sizeof(float) * 2 * c.nv * kMaxInstances)) != cudaSuccess ||
+        (e = cudaMalloc(&c.slopes, sizeof(float) * 2 * c.nv * kMaxInstances * 2)) != cudaSuccess ||
         (e = cudaMalloc(&c.layers, sizeof(float) * SS * kMaxInstances)) != cudaSuccess ||
         (e = cudaMalloc(&c.work, sizeof(int) * 4)) != cudaSuccess)
         return bail(e, "calibration scratch");
@@ -2375,7 +2375,11 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
     const SpotGroup &G = h->groups[c.group];
     const size_t SS = (size_t)h->S * h->S;
     const int n_slopes = 2 * c.nv;
-    const int per_chunk = kMaxInstances / 2;
+    // The 32-point tensor-core kernels measure a mode and its negative from one wavefront (the negated
+    // wavefront's spot is the spot mirrored), 64 modes a chunk; other kernels take them as two
+    // instances, 32 modes a chunk.
+    const bool pairs = is_tc(c.kind) && h->geoms[c.geom].g.n_fft == 32;
+    const int per_mode = pairs ? 1 : 2, per_chunk = kMaxInstances / per_mode;
     static thread_local DmLayerBatch batch;
     static thread_local ProjArgs pa;
     static thread_local ShArgs sa;
@@ -2388,12 +2392,13 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             c.cur_dm = (int)d;
         }
         for (int m0 = 0; m0 < M.d.n_modes; m0 += per_chunk) {
-            const int K = std::min(per_chunk, M.d.n_modes - m0), ni = 2 * K;
-            // instance 2k: +amplitude of mode m0 + k in the beam (coefficient -amplitude), 2k + 1: -amplitude
+            const int K = std::min(per_chunk, M.d.n_modes - m0), ni = per_mode * K;
+            // +amplitude of mode m0 + k in the beam (coefficient -amplitude): instance k of pairs, else 2k,
+            // and -amplitude 2k + 1
             batch.n = ni;
             for (int i = 0; i < ni; ++i)
-                batch.l[i] = dm_layer_args(h, M, M.d.m2a + m0 + i / 2, M.d.n_modes,
-                                           (float)((i & 1) ? amplitude : -amplitude), c.layers + i * SS);
+                batch.l[i] = dm_layer_args(h, M, M.d.m2a + m0 + i / per_mode, M.d.n_modes,
+                                           (float)(i % per_mode ? amplitude : -amplitude), c.layers + i * SS);
             long sl = timed_begin(h, "dm_layer", s);
             e = launch_dm_layers(batch, s);
             timed_end(h, sl, s);
@@ -2413,7 +2418,7 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             for (int i = 0; i < ni; ++i) {
                 dyn.dm = c.layers + i * SS;
                 dyn.opd = c.opd + i * c.opd_stride;
-                dyn.slopes = c.slopes + (size_t)i * n_slopes;
+                dyn.slopes = c.slopes + (size_t)i * (3 - per_mode) * n_slopes;  // row 2k of mode k, then 2k + 1
                 pa.dyn[i] = dyn;
             }
             sl = timed_begin(h, "project", s);
@@ -2432,6 +2437,7 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             sa.n_inst = ni;
             sa.work = c.work + 2;
             sa.project = 0;
+            sa.pair_off = pairs ? n_slopes : 0;
             memcpy(sa.dyn, pa.dyn, sizeof(InstDyn) * ni);  // no noise: the spot kernel takes the centroids
             sl = timed_begin(h, kind_name(c.kind) + std::to_string(sa.N), s);
             e = launch_spot(c.kind, sa, s, !h->timing);

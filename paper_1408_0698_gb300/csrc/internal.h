@@ -141,6 +141,9 @@ struct ShArgs {
     // LGS per-slice model on kernels that read projected slices: slice s of a subaperture's OPD
     // sits s * slice_opd_stride floats after slice 0; 0 = one OPD
     long long slice_opd_stride;
+    // 32-point tensor-core kernels, push-pull pairs: the slopes of the negated wavefront too, pair_off
+    // floats after those of the wavefront (no noise, no stage outputs); 0 = off
+    long long pair_off;
     int split_noise;     // 32-point kernels: 1 = store the expected image (dyn.st_E, required)
                          // and stop; launch_noise_cog completes the measurement; 0 = no instance
                          // has noise on: the centroid of the expected image in the spot kernel

@@ -175,7 +175,7 @@ struct TcLayout {
 
 }  // namespace
 
-template <int n, int N, int nd, bool kF16, bool kMmaU, int WG>
+template <int n, int N, int nd, bool kF16, bool kMmaU, int WG, bool kPair>
 __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __grid_constant__ ShArgs a) {
     using Lay = TcLayout<n, N, nd, false, kMmaU, WG>;
     // warpgroups per CTA (the tile shape the tuner picks): their threads and tensor-memory columns
@@ -512,11 +512,43 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
 
         // remaining stages on the CUDA cores (per warp)
         float Bv[nd / 2];
-        if (W.is_lgs) {
-            tail::lgs_binned<n, nd>(T, Bw, fft, a.Gc, kq, lane, Bv);
-        } else
-            tail::ngs_binned<nd>(Iw, lane, Bv);
-        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
+        float *slopes = D.slopes + W.slope_off;
+        if constexpr (kPair) {
+            // the wavefront, then its negative: the spot mirrored, so the conjugate transfer-domain
+            // image (LGS) or the slopes' negatives (NGS)
+            if (W.is_lgs) {
+                float2 Tr[n / 2], Ti[n / 2];
+                tail::lane_dft<n>(T, fft, lane, Tr, Ti);
+#pragma unroll 1
+                for (int s = 0; s < 2; ++s) {
+                    const float2 sg = tail::dup2(s ? -1.0f : 1.0f);
+                    float2 Ur[n / 2], Ui[n / 2];
+#pragma unroll
+                    for (int c = 0; c < n / 2; ++c) {
+                        Ur[c] = Tr[c];
+                        Ui[c] = tail::mul2(Ti[c], sg);
+                    }
+                    tail::lgs_binned<n, nd>(Ur, Ui, fft[(s ? 10 : 5) * 32 + lane], Bw, fft, a.Gc, kq, lane, Bv);
+                    tail::finish<nd>(Bv, W, D, v, lane, false, slopes + (s ? a.pair_off : 0));
+                }
+            } else {
+                tail::ngs_binned<nd>(Iw, lane, Bv);
+                tail::finish<nd>(Bv, W, D, v, lane, false, slopes);
+                if (lane == 0) {
+                    slopes[a.pair_off + 2 * v] = -slopes[2 * v];
+                    slopes[a.pair_off + 2 * v + 1] = -slopes[2 * v + 1];
+                }
+            }
+        } else {
+            if (W.is_lgs) {
+                float2 Tr[n / 2], Ti[n / 2];
+                tail::lane_dft<n>(T, fft, lane, Tr, Ti);
+                tail::lgs_binned<n, nd>(Tr, Ti, fft[5 * 32 + lane], Bw, fft, a.Gc, kq, lane, Bv);
+            } else {
+                tail::ngs_binned<nd>(Iw, lane, Bv);
+            }
+            tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0, slopes);
+        }
     }
     fence_before_sync();
     __syncthreads();
@@ -834,10 +866,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         // remaining stages on the CUDA cores (per warp)
         float Bv[nd / 2];
         if (W.is_lgs) {
-            tail::lgs_binned<n, nd>(T, Bw, fft, a.Gc, kq, lane, Bv);
+            float2 Tr[n / 2], Ti[n / 2];
+            tail::lane_dft<n>(T, fft, lane, Tr, Ti);
+            tail::lgs_binned<n, nd>(Tr, Ti, fft[5 * 32 + lane], Bw, fft, a.Gc, kq, lane, Bv);
         } else
             tail::ngs_binned<nd>(Iw, lane, Bv);
-        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0);
+        tail::finish<nd>(Bv, W, D, v, lane, a.split_noise != 0, D.slopes + W.slope_off);
     }
     fence_before_sync();
     __syncthreads();
@@ -900,12 +934,12 @@ float bf16_float(uint16_t h) {
     return f;
 }
 
-template <int n, int N, int nd, bool kSlices, bool kF16, bool kMmaU, int WG = kWG>
+template <int n, int N, int nd, bool kSlices, bool kF16, bool kMmaU, int WG = kWG, bool kPair = false>
 cudaError_t shape_tc_k(const ShArgs &a, LaunchShape *out) {
     using Lay = TcLayout<n, N, nd, kSlices, kSlices ? false : kMmaU, WG>;
     const void *f;
     if constexpr (kSlices) f = (const void *)k_sh_tc_sl<n, nd, kF16>;
-    else f = (const void *)k_sh_tc<n, N, nd, kF16, kMmaU, WG>;
+    else f = (const void *)k_sh_tc<n, N, nd, kF16, kMmaU, WG, kPair>;
     const int smem = Lay::bytes;  // no static shared memory: the dynamic base is 1024-aligned
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -930,6 +964,9 @@ template <int n, int N, int nd>
 cudaError_t shape_tc(const ShArgs &a, LaunchShape *out, bool f16) {
     if (a.slice_opd_stride > 0)
         return f16 ? shape_tc_k<n, N, nd, true, true, false>(a, out) : shape_tc_k<n, N, nd, true, false, false>(a, out);
+    if (a.pair_off > 0)
+        return f16 ? shape_tc_k<n, N, nd, false, true, false, kWG, true>(a, out)
+                   : shape_tc_k<n, N, nd, false, false, false, kWG, true>(a, out);
     if (a.mma_u)
         return f16 ? shape_tc_k<n, N, nd, false, true, true>(a, out) : shape_tc_k<n, N, nd, false, false, true>(a, out);
     // ShArgs::cta_warps = 4: one warpgroup per CTA (else two)

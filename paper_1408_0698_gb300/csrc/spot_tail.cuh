@@ -35,13 +35,14 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-constexpr int kFftTable = 10 * 32;  // float2: five stages of twiddles, ph h(dy), four more stages
+constexpr int kFftTable = 11 * 32;  // float2: five stages of twiddles, ph h(dy), four more stages, ph* h(dy)
 
 // Per-lane DFT constants: entry s * 32 + lane (s < 5, span h = 16 >> s) is 1 for the upper
 // lane of a butterfly and w^((lane mod h) 16 / h) for the lower; entry 5 * 32 + lane is
 // ph(dy) h(dy) = sum_{r<2} exp(-2 pi i r dy / 32) of the lane's output frequency dy when
 // |dy| < n, else 0; entry (6 + s) * 32 + lane (s < 4, span q = 2^s in positions p = lane >> 1)
-// is 1 for the upper position of a butterfly and exp(-2 pi i (p mod q) / 2q) for the lower.
+// is 1 for the upper position of a butterfly and exp(-2 pi i (p mod q) / 2q) for the lower; entry
+// 10 * 32 + lane is ph(dy)* h(dy) = sum_{r<2} exp(-2 pi i (r + 1) dy / 32) for |dy| < n, else 0.
 // Call from every thread of the block.
 template <int n>
 __device__ __forceinline__ void fill_fft_table(float2 *tab, int tid, int nthreads) {
@@ -59,9 +60,19 @@ __device__ __forceinline__ void fill_fft_table(float2 *tab, int tid, int nthread
             } else {
                 cs = 0.0f;
             }
-        } else {
+        } else if (st < 10) {
             const int q = 1 << (st - 6), p = l >> 1;
             if (p & q) sincospif((float)(-(p & (q - 1))) / (float)q, &sn, &cs);
+        } else {
+            const int f = (int)(__brev((unsigned)l) >> 27), dy = f < 16 ? f : f - 32;
+            cs = 0.0f;
+            if (dy > -n && dy < n) {
+                float s1, c1, s2, c2;
+                sincospif((float)(-dy) / 16.0f, &s1, &c1);
+                sincospif((float)(-2 * dy) / 16.0f, &s2, &c2);
+                sn = s1 + s2;
+                cs = c1 + c2;
+            }
         }
         tab[i] = make_float2(cs, sn);
     }
@@ -86,20 +97,16 @@ __device__ __forceinline__ void load_ktil(const float2 *kt, int lane, float4 (&k
 
 constexpr int kBScratch = 272;  // floats: the 16 x 16 image, its lower half 16 words off
 
-// T: this lane's row k = lane of the first stage (T[k][dx], dx < n), consumed.  fft: the
-// table above.  kq: load_ktil.  Gc: uniform G for ix < nd/2, entry ix (n/2) + c holds the columns
-// dx = 2c, 2c + 1 as (re, re, -im, -im) (ShArgs::Gc).  Bs is per-warp scratch (kBScratch floats,
-// 16-byte aligned).
-// On return Bv[j] = B[half * nd/2 + j][ix] for lane = half * 16 + ix.
-template <int n, int nd>
-__device__ __forceinline__ void lgs_binned(float2 (&T)[n], float *Bs, const float2 *fft, const float4 *Gc,
-                                           const float4 (&kq)[n / 2], int lane, float (&Bv)[nd / 2]) {
-    constexpr int P = n / 2, PH = (P + 1) / 2;
-    static_assert(nd == 16, "the detector tile maps to 16 lanes x 2 half-warps");
+// The first part of the elongation stage.  T: this lane's row k = lane of the first stage (T[k][dx],
+// dx < n); on return Tr[c], Ti[c] are the parts of sum_k w^(k dy) T[k][dx] for the lane's frequency dy
+// and the columns dx = 2c, 2c + 1.  fft: the table above.
+template <int n>
+__device__ __forceinline__ void lane_dft(const float2 (&T)[n], const float2 *fft, int lane, float2 (&Tr)[n / 2],
+                                         float2 (&Ti)[n / 2]) {
+    constexpr int P = n / 2;
     static_assert(n <= 16, "frequencies |dy| < n must be distinct modulo 32");
     static_assert(n % 2 == 0, "columns travel in pairs");
     // columns as pairs: Tr[c] = (re 2c, re 2c+1), Ti[c] = (im 2c, im 2c+1)
-    float2 Tr[P], Ti[P];
 #pragma unroll
     for (int c = 0; c < P; ++c) {
         Tr[c] = make_float2(T[2 * c].x, T[2 * c + 1].x);
@@ -123,10 +130,23 @@ __device__ __forceinline__ void lgs_binned(float2 (&T)[n], float *Bs, const floa
             Ti[c] = fma2(si, twx, mul2(sr, twy));
         }
     }
+}
+
+// The rest, from lane_dft's Tr, Ti (consumed).  ph: the lane's entry 5 of the table; with Ti negated and
+// entry 10 instead, the stage takes the conjugate of the spot's transfer-domain image, which is that
+// of the spot mirrored about its centre: the spot of the negated wavefront.  kq: load_ktil.  Gc:
+// uniform G for ix < nd/2, entry ix (n/2) + c holds the columns dx = 2c, 2c + 1 as (re, re, -im, -im)
+// (ShArgs::Gc).  Bs is per-warp scratch (kBScratch floats, 16-byte aligned).
+// On return Bv[j] = B[half * nd/2 + j][ix] for lane = half * 16 + ix.
+template <int n, int nd>
+__device__ __forceinline__ void lgs_binned(float2 (&Tr)[n / 2], float2 (&Ti)[n / 2], const float2 ph, float *Bs,
+                                           const float2 *fft, const float4 *Gc, const float4 (&kq)[n / 2], int lane,
+                                           float (&Bv)[nd / 2]) {
+    constexpr int P = n / 2, PH = (P + 1) / 2;
+    static_assert(nd == 16, "the detector tile maps to 16 lanes x 2 half-warps");
     // h(dy) M[dy] for the lane's frequency (zero outside the band |dy| < n, through the table),
     // then folded with the lane holding dy -/+ 16
     {
-        const float2 ph = fft[5 * 32 + lane];
         const float2 phx = dup2(ph.x), phy = dup2(ph.y), nphy = dup2(-ph.y);
 #pragma unroll
         for (int c = 0; c < P; ++c) {
@@ -381,13 +401,13 @@ __device__ __forceinline__ void noise_centroid(const float (&ev)[nd / 2], const 
 }
 
 // Photometry, then the centroid of the expected image in place (a measurement without noise); with
-// split, the expected image is stored and the noise kernel completes the measurement.  The sums of
+// split, the expected image is stored and the noise kernel completes the measurement.  slopes: the WFS's.  The sums of
 // the centroid run in noise_centroid's order.  Without noise the image would only travel to the
 // noise kernel and back: ELT frame, FP32, 125.5 us + 17.2 us for that pass -> 129.4 us in place
 // (the frame 181.5 -> 172.7 us); a calibration's chunk of 64 measurements 857 + 148 us -> 869 us.
 template <int nd>
 __device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc &W, const InstDyn &D, int v,
-                                       int lane, bool split) {
+                                       int lane, bool split, float *slopes) {
     constexpr int nd2 = nd * nd, J = nd / 2;
     const int ix = lane & 15, half = lane >> 4;
     float ev[J];
@@ -410,9 +430,8 @@ __device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc 
     sy = warp_sum(sy);
     if (lane == 0) {
         const bool ok = sc > 0.0f;
-        float *sl = D.slopes + W.slope_off;
-        sl[2 * v] = ok ? sx / sc : 0.0f;
-        sl[2 * v + 1] = ok ? sy / sc : 0.0f;
+        slopes[2 * v] = ok ? sx / sc : 0.0f;
+        slopes[2 * v + 1] = ok ? sy / sc : 0.0f;
     }
 }
 
