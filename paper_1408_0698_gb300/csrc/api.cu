@@ -2380,7 +2380,6 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
     // instances, 32 modes a chunk.
     const bool pairs = is_tc(c.kind) && h->geoms[c.geom].g.n_fft == 32;
     const int per_mode = pairs ? 1 : 2, per_chunk = kMaxInstances / per_mode;
-    static thread_local DmLayerBatch batch;
     static thread_local ProjArgs pa;
     static thread_local ShArgs sa;
     cudaError_t e;
@@ -2395,12 +2394,9 @@ wfs_status wfs_loop_calibrate(wfs_loop lp, int gs, double amplitude, float *im_o
             const int K = std::min(per_chunk, M.d.n_modes - m0), ni = per_mode * K;
             // +amplitude of mode m0 + k in the beam (coefficient -amplitude): instance k of pairs, else 2k,
             // and -amplitude 2k + 1
-            batch.n = ni;
-            for (int i = 0; i < ni; ++i)
-                batch.l[i] = dm_layer_args(h, M, M.d.m2a + m0 + i / per_mode, M.d.n_modes,
-                                           (float)(i % per_mode ? amplitude : -amplitude), c.layers + i * SS);
             long sl = timed_begin(h, "dm_layer", s);
-            e = launch_dm_layers(batch, s);
+            e = launch_dm_modes(dm_layer_args(h, M, M.d.m2a + m0, M.d.n_modes, (float)-amplitude, c.layers), K, per_mode,
+                                SS, s);
             timed_end(h, sl, s);
             if (e != cudaSuccess) return cuda_fail(h, e, "calibration layers");
             InstDyn dyn;

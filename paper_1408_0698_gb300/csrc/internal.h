@@ -316,6 +316,10 @@ struct DmLayerBatch {
     DmLayerArgs l[kMaxInstances];
 };
 cudaError_t launch_dm_layers(const DmLayerBatch &b, cudaStream_t s);
+// Layers of n_modes consecutive columns of the modal base a.act (a.act_stride apart per actuator): for
+// each mode a.act_scale times the mode and, with per_mode = 2, its negative, `stride` floats apart from
+// a.layer on.
+cudaError_t launch_dm_modes(const DmLayerArgs &a, int n_modes, int per_mode, size_t stride, cudaStream_t s);
 // IM rows of a push-pull chunk: im[k][j] = (s[2k][j] - s[2k+1][j]) / (2 amplitude) for k < n_modes,
 // j < n_slopes, instance i's slopes at s + i * n_slopes.
 cudaError_t launch_push_pull_rows(const float *s, int n_modes, int n_slopes, float inv_2a, float *im,

@@ -165,18 +165,35 @@ cudaError_t launch_gemv(const GemvArgs &a, cudaStream_t s) { return launch_gemv_
 // get weight zero (their index is clamped to a valid one).  The actuator pitch is at least the
 // screen pitch, so the tile's 64 rows reach at most 64 + 2R + 2 actuator rows.
 //
-// The tile's actuators are read once into shared memory, kDmChunk actuator rows at a time (a modal-base
-// column's are n_modes apart: a sector each), and in the second pass a warp owns 8 consecutive rows and
-// keeps their column of T in registers while the rows' first actuator stays the same.
-// Bound: latency of the strided reads.  64 layers of 800 x 800 pixels of a 5,000-mode base: 161 us
-// with every tap read from global memory and T from shared memory per row -> DMTIME us.
+// A CTA takes its tile for kM consecutive modes (columns of a modal base, neighbours in memory): the
+// tile's weights are formed once, and two modes at a time share every weight as the halves of a packed
+// FP32 pair.  NW = 2R + 2 is unrolled; the actuators are read once into shared memory, and in the
+// second pass a warp owns 8 consecutive rows and keeps their column of T in registers while the rows'
+// first actuator stays the same.
+// Bound: issue slots, then the writes (3 MB a layer).  64 layers of 860 x 860 pixels of a 5,000-mode
+// base: 181 us with a tile per layer, weight by weight (127 instructions a pixel) -> 74.5 us; the three
+// layers of an ELT loop step 17.1 -> 16.5 us.
 namespace {
 constexpr int kDmTx = 32, kDmTy = 64;
 constexpr int kDmW = 2 * kMaxDmSupport + 2;     // weights per pixel and axis
 constexpr int kDmRows = kDmTy + kDmW;           // actuator rows a tile reaches
 constexpr int kDmCols = kDmTx + kDmW;           // actuator columns a tile reaches
-constexpr int kDmChunk = 16;                    // actuator rows staged at a time
-}
+constexpr int kDmModes = 8;                     // modes per tile of a calibration
+constexpr int kDmStage = 4800;                  // staged actuators: all rows of a usual tile, or in parts
+static_assert(kDmStage >= kDmCols * kDmModes, "at least one actuator row is staged");
+
+struct DmSmem {
+    float cw[kDmTx][kDmW + 1];
+    alignas(16) float rw[kDmTy][20];
+    alignas(16) float act[kDmStage];            // [row][column][mode]
+    float2 T[kDmRows][kDmTx];
+    int cb[kDmTx], rb[kDmTy];
+};
+
+// The kernel body of a support (1 .. 8), by its weights per axis.
+#define GBWFS_DM_SUPPORTS(CASE) CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
+static_assert(kMaxDmSupport == 8, "a case for every support");
+}  // namespace
 
 __device__ __forceinline__ void dm_axis_weights(const DmLayerArgs &a, int pix, int &base, float *w) {
     int off;
@@ -192,59 +209,120 @@ __device__ __forceinline__ void dm_axis_weights(const DmLayerArgs &a, int pix, i
     }
 }
 
-// blockIdx.z: the layer of the batch; the grid covers the largest window, CTAs past a smaller
-// one leave at once.
-__global__ void __launch_bounds__(256) k_dm_layer(const __grid_constant__ DmLayerBatch b) {
-    __shared__ float cw[kDmTx][kDmW + 1], rw[kDmTy][kDmW], T[kDmRows][kDmTx], act[kDmChunk][kDmCols];
-    __shared__ int cb[kDmTx], rb[kDmTy];
-    const DmLayerArgs &a = b.l[blockIdx.z];
+// Modes 0 .. modes - 1 (at most kM): per mode the layer of act_scale times the mode and, with
+// per_mode = 2, its negative, `stride` floats after each other.
+template <int NW, int kM>
+__device__ __forceinline__ void dm_tile(const DmLayerArgs &a, int m0, int modes, int per_mode, size_t stride, DmSmem &sm) {
+    static_assert(kM % 2 == 0 && NW <= kDmW && kDmW <= 20, "row weights in whole 16-byte words");
     if ((int)blockIdx.x * kDmTx >= a.w || (int)blockIdx.y * kDmTy >= a.h) return;
     const int j0 = a.x0 + blockIdx.x * kDmTx, i0 = a.y0 + blockIdx.y * kDmTy;
-    const int nw = 2 * a.support + 2;
-    const int t = threadIdx.x;
+    auto &[cw, rw, act, T, cb, rb] = sm;
+    const int t = threadIdx.x, warp = t >> 5, jj = t & 31, j = j0 + jj;
     if (t < kDmTx) dm_axis_weights(a, j0 + t, cb[t], cw[t]);
     else if (t < kDmTx + kDmTy) dm_axis_weights(a, i0 + t - kDmTx, rb[t - kDmTx], rw[t - kDmTx]);
     __syncthreads();
-    // pass 1: the actuator rows ay_lo .. ay_lo + nr - 1 the tile's rows reach, their columns
-    // ax_lo .. ax_lo + nc - 1 (clamped to the grid)
-    const int ay_lo = rb[0], ax_lo = cb[0];
-    const int nr = min(rb[kDmTy - 1] + nw - ay_lo, kDmRows), nc = min(cb[kDmTx - 1] + nw - ax_lo, kDmCols);
-    for (int c0 = 0; c0 < nr; c0 += kDmChunk) {
-        const int rows = min(kDmChunk, nr - c0);
-        for (int e = t; e < rows * nc; e += 256) {
-            const int r = e / nc, c = e - r * nc, ay = ay_lo + c0 + r, ax = min(max(ax_lo + c, 0), a.n_act - 1);
-            act[r][c] = ay >= 0 && ay < a.n_act ? __ldg(a.act + ((size_t)ay * a.n_act + ax) * a.act_stride) : 0.0f;
-        }
-        __syncthreads();
-        for (int e = t; e < rows * kDmTx; e += 256) {
-            const int r = e / kDmTx, jj = e - r * kDmTx, c = cb[jj] - ax_lo;
-            float acc = 0.0f;
-            for (int k = 0; k < nw; ++k) acc = fmaf(act[r][c + k], cw[jj][k], acc);
-            T[c0 + r][jj] = acc * a.act_scale;
-        }
-        __syncthreads();
-    }
-    // pass 2: one column per lane, 8 consecutive rows per warp
-    const int jj = t & 31, j = j0 + jj;
-    if (j >= a.x0 + a.w) return;
-    float tc[kDmW];
-    int have = -1;
-    for (int ii = (t >> 5) * 8; ii < (t >> 5) * 8 + 8; ++ii) {
-        const int i = i0 + ii;
-        if (i >= a.y0 + a.h) break;
-        const int r0 = rb[ii] - ay_lo;
-        if (r0 != have) {
+    const int ay_lo = rb[0], ax_lo = cb[0], col = cb[jj] - ax_lo;
+    const int nr = min(rb[kDmTy - 1] + NW - ay_lo, kDmRows), nc = min(cb[kDmTx - 1] + NW - ax_lo, kDmCols);
+    const int chunk = kDmStage / (nc * kM);  // actuator rows staged at a time
+    const bool one = nr <= chunk;            // the actuators of all modes stay in shared memory
+    float w1[NW];
 #pragma unroll
-            for (int k = 0; k < kDmW; ++k)
-                if (k < nw) tc[k] = T[r0 + k][jj];
-            have = r0;
-        }
-        float sum = 0.0f;
+    for (int k = 0; k < NW; ++k) w1[k] = cw[jj][k];
+    for (int m = 0; m < modes; m += 2) {
+        for (int c0 = 0; c0 < nr; c0 += chunk) {
+            const int rows = min(chunk, nr - c0);
+            if (m == 0 || !one) {
+                for (int e = t; e < rows * nc * kM; e += 256) {
+                    const int q = e % kM, rc = e / kM, r = rc / nc, c = rc - r * nc;
+                    const int ay = ay_lo + c0 + r, ax = min(max(ax_lo + c, 0), a.n_act - 1);
+                    act[e] = ay >= 0 && ay < a.n_act && q < modes
+                                 ? __ldg(a.act + ((size_t)ay * a.n_act + ax) * a.act_stride + m0 + q)
+                                 : 0.0f;
+                }
+                __syncthreads();
+            }
+            for (int r = warp; r < rows; r += 8) {
+                const float2 *src = reinterpret_cast<const float2 *>(act + (r * nc + col) * kM + m);
+                float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll
-        for (int k = 0; k < kDmW; ++k)
-            if (k < nw) sum = fmaf(rw[ii][k], tc[k], sum);
-        a.layer[(size_t)i * a.S + j] = -sum;  // the mirror takes its shape out of the beam
+                for (int k = 0; k < NW; ++k)
+                    acc = __ffma2_rn(src[k * (kM / 2)], make_float2(w1[k], w1[k]), acc);
+                T[c0 + r][jj] = make_float2(acc.x * a.act_scale, acc.y * a.act_scale);
+            }
+            __syncthreads();
+        }
+        // one column per lane, 8 consecutive rows per warp
+        const bool second = m + 1 < modes;
+        float *la = a.layer + (size_t)(m0 + m) * per_mode * stride + j;
+        float *lb = la + per_mode * stride;
+        float2 tc[NW];
+        int have = -1;
+        for (int ii = warp * 8; ii < warp * 8 + 8; ++ii) {
+            const int i = i0 + ii;
+            if (i >= a.y0 + a.h) break;
+            const int r0 = rb[ii] - ay_lo;
+            if (r0 != have) {
+#pragma unroll
+                for (int k = 0; k < NW; ++k) tc[k] = T[r0 + k][jj];
+                have = r0;
+            }
+            float2 sum = make_float2(0.0f, 0.0f);
+            const float4 *w4 = reinterpret_cast<const float4 *>(rw[ii]);
+#pragma unroll
+            for (int k = 0; k < NW; k += 4) {
+                const float4 w = w4[k / 4];
+                sum = __ffma2_rn(tc[k], make_float2(w.x, w.x), sum);
+                if (k + 1 < NW) sum = __ffma2_rn(tc[k + 1], make_float2(w.y, w.y), sum);
+                if (k + 2 < NW) sum = __ffma2_rn(tc[k + 2], make_float2(w.z, w.z), sum);
+                if (k + 3 < NW) sum = __ffma2_rn(tc[k + 3], make_float2(w.w, w.w), sum);
+            }
+            if (j < a.x0 + a.w) {
+                const size_t o = (size_t)i * a.S;
+                la[o] = -sum.x;  // the mirror takes its shape out of the beam
+                if (second) lb[o] = -sum.y;
+                if (per_mode == 2) {
+                    la[stride + o] = sum.x;
+                    if (second) lb[stride + o] = sum.y;
+                }
+            }
+        }
+        __syncthreads();  // T is rewritten for the next modes
     }
+}
+
+// blockIdx.z: the layer of the batch; the grid covers the largest window, CTAs past a smaller
+// one leave at once.
+__global__ void __launch_bounds__(256) k_dm_layer(const __grid_constant__ DmLayerBatch b) {
+    __shared__ DmSmem sm;
+    const DmLayerArgs &a = b.l[blockIdx.z];
+    switch (a.support) {
+#define GBWFS_DM_CASE(R) \
+    case R: dm_tile<2 * R + 2, 2>(a, 0, 1, 1, 0, sm); break;
+        GBWFS_DM_SUPPORTS(GBWFS_DM_CASE)
+#undef GBWFS_DM_CASE
+    }
+}
+
+// The layers of consecutive modes of one modal base over the same window (a calibration's chunk).
+template <int NW>
+__global__ void __launch_bounds__(256) k_dm_modes(const __grid_constant__ DmLayerArgs a, int n_modes, int per_mode,
+                                                  size_t stride) {
+    __shared__ DmSmem sm;
+    const int m0 = blockIdx.z * kDmModes;
+    dm_tile<NW, kDmModes>(a, m0, min(kDmModes, n_modes - m0), per_mode, stride, sm);
+}
+
+cudaError_t launch_dm_modes(const DmLayerArgs &a, int n_modes, int per_mode, size_t stride, cudaStream_t s) {
+    if (n_modes <= 0 || a.w == 0 || a.h == 0) return cudaSuccess;
+    if (a.support < 1 || a.support > kMaxDmSupport || !(a.r_hi <= 1.0f) || a.w < 0 || a.h < 0) return cudaErrorInvalidValue;
+    const dim3 grid((a.w + kDmTx - 1) / kDmTx, (a.h + kDmTy - 1) / kDmTy, (n_modes + kDmModes - 1) / kDmModes);
+    switch (a.support) {
+#define GBWFS_DM_CASE(R) \
+    case R: k_dm_modes<2 * R + 2><<<grid, 256, 0, s>>>(a, n_modes, per_mode, stride); break;
+        GBWFS_DM_SUPPORTS(GBWFS_DM_CASE)
+#undef GBWFS_DM_CASE
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_dm_layers(const DmLayerBatch &b, cudaStream_t s) {
