@@ -1060,6 +1060,7 @@ wfs_status wfs_create(const wfs_telescope *tel, int n_gs, const wfs_guide_star *
             memset(&ka, 0, sizeof ka);
             ka.subap = s.d_ids;
             ka.ktil = s.d_ktil;
+            ka.pairs = runs_tc(g) ? 1 : 0;
             ka.n = n;
             ka.N = g.n_fft;
             ka.n_sub = g.n_sub;
@@ -2138,8 +2139,9 @@ wfs_status wfs_batch_tune(wfs_batch b, const float *const *screens, const double
         } else if (is_tc(bc.kind) && bc.geom->g.n_fft == 64) {
             for (int m : {1, 2}) cand.push_back({76 * m, 0});
         } else if (is_tc(bc.kind)) {
-            // tile shape: two warpgroups (8 subapertures) per CTA, at most 2 CTAs per SM, or one
-            // (4 subapertures) with up to 3 CTAs per SM; and the persistent grid size
+            // tile shape: six warpgroups (24 subapertures) per CTA, one CTA per SM, or two (8), at most
+            // 2 CTAs per SM, or one (4) with up to 3 CTAs per SM; and the persistent grid size
+            cand.push_back({152, 24});
             for (int m : {1, 2}) cand.push_back({152 * m, 8});
             for (int m : {1, 2, 3}) cand.push_back({152 * m, 4});
         } else {
@@ -2511,6 +2513,7 @@ wfs_status wfs_set_lgs_model(wfs_handle h, int per_slice) {
             memset(&ka, 0, sizeof ka);
             ka.subap = G.d_ids;
             ka.ktil = G.d_ktil_g;
+            ka.pairs = runs_tc(geo) ? 1 : 0;
             ka.n = n;
             ka.N = geo.n_fft;
             ka.n_sub = geo.n_sub;

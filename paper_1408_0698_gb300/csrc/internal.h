@@ -63,7 +63,7 @@ struct WfsDesc {                    // static per wavefront sensor
     const int32_t *subap;           // [n_valid] ids sy * n_sub + sx
     const uint32_t *mask;           // [n_valid][mask_words] lit-pixel bits, bit p*n+q
     const float *fill;              // [n_valid]
-    const float2 *ktil;             // [n_valid][(2n-1)*n] elongation transfer (LGS only)
+    const float2 *ktil;             // [n_valid][(2n-1)*n] elongation transfer (LGS only; KtilArgs::pairs)
     long long opd_off, slope_off, int_off, det_off;  // into the instance's buffers (floats)
     // first whole-width and first narrow projection block of this WFS among its launch's (place_blocks)
     int proj_block_begin, proj_part_begin;
@@ -155,6 +155,7 @@ struct KtilArgs {
     const int32_t *subap;
     float2 *ktil;
     int n, N, n_sub, n_valid, n_na;
+    int pairs;  // layout of a subaperture's table: 0 [2n-1][n]; 1 column pairs first, [n/2][2n-1][2]
     double D, dx, pix_rad, sigma_px, launch_x, launch_y, h0;
     double alt[kMaxNaSlices], w[kMaxNaSlices];
 };

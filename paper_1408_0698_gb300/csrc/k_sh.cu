@@ -429,7 +429,8 @@ __global__ void __launch_bounds__(128) k_ktil(const __grid_constant__ KtilArgs a
             im += a.w[s] * (p.x * q.y + p.y * q.x);
         }
         const double c = (dx == 0 ? 1.0 : 2.0) / ((double)N * N * s_norm);
-        a.ktil[(size_t)v * D2 * n + o] = make_float2((float)(re * c), (float)(im * c));
+        const int at = a.pairs ? ((dx >> 1) * D2 + dyi) * 2 + (dx & 1) : o;
+        a.ktil[(size_t)v * D2 * n + at] = make_float2((float)(re * c), (float)(im * c));
     }
 }
 

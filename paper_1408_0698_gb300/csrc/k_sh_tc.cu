@@ -27,10 +27,11 @@
 // from the kernel parameters, the rows of Q stay in registers, K~ goes from global memory to registers
 // under the second product and the field is written as whole 16-byte entries: 640 -> 558 wavefronts and
 // 1,684 -> 1,557 warp instructions per LGS subaperture, ELT frame (27,792 of them) 94.3 -> 88.8 us, the
-// same bits.
+// same bits.  K~ is stored with column pairs first, so that a warp reads 512 contiguous bytes where
+// rows of n put a lane's word into a sector of its own: 86.3 us.
 //
-// CTA = two warpgroups (4 warps each); warp w of a warpgroup owns subaperture 4g + w of its
-// group g and its lane k owns DFT row k, which is also TMEM lane 32 w + k of both accumulators.
+// CTA = two warpgroups (4 warps each), or six in launches of many subapertures (shape_tc); warp w of a
+// warpgroup owns subaperture 4g + w of its group g and its lane k owns DFT row k, which is also TMEM lane 32 w + k of both accumulators.
 //
 // The per-slice variant (k_sh_tc_sl, launched with ShArgs::slice_opd_stride) runs the LGS
 // per-slice model (Sec. 4: one wavefront and one spot per sodium sub-layer, piled up with the
@@ -176,11 +177,15 @@ struct TcLayout {
 }  // namespace
 
 template <int n, int N, int nd, bool kF16, bool kMmaU, int WG, bool kPair>
-__global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __grid_constant__ ShArgs a) {
+__global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : WG == 2 ? 2 : 1) k_sh_tc(const __grid_constant__ ShArgs a) {
     using Lay = TcLayout<n, N, nd, false, kMmaU, WG>;
-    // warpgroups per CTA (the tile shape the tuner picks): their threads and tensor-memory columns
+    // warpgroups per CTA (the tile shape): their threads and tensor-memory columns
     constexpr int kWG = WG, kTcThreads = 128 * WG;
-    constexpr uint32_t kTmemCols = 128 * WG;
+    // Y's 64 columns, then Ta's 32 in the same place (Y has been read by then); U's 128 columns where
+    // it is an MMA; allocations are powers of two
+    constexpr uint32_t kCols = kMmaU ? 128 : 64;
+    constexpr uint32_t kTmemCols = kCols * WG <= 64 ? 64 : kCols * WG <= 128 ? 128 : kCols * WG <= 256 ? 256 : 512;
+    constexpr uint32_t kTa = kMmaU ? 64 : 0;
     using E = TcElt<kF16>;
     constexpr int D2 = Lay::D2, nd2 = nd * nd;
     static_assert(6 * n <= 64 && n <= 16, "the split DFT operand must fit one 64-element K atom");
@@ -246,7 +251,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
     const uint32_t tmem_all = *tslot;
     wait_prior_grid();
     if (a.split_noise) allow_dependent_grid();  // the noise kernel may take SMs as CTAs retire
-    const uint32_t tmem = tmem_all + 128u * wg;  // this warpgroup's columns
+    const uint32_t tmem = tmem_all + kCols * wg;  // this warpgroup's columns
     const uint32_t t_row = tmem + ((uint32_t)(wq * 32) << 16);
     constexpr uint32_t idesc1 = tc_idesc(128, 64, E::fmt), idesc2 = tc_idesc(128, 32, E::fmt);
     constexpr uint32_t idesc0 = tc_idesc(128, 128, E::fmt);
@@ -483,10 +488,10 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         if (issuer) {
 #pragma unroll
             for (int s = 0; s < 4; ++s)
-                mma_f16(tmem + 64, sw128_desc(smem_u32(sA2) + 32 * s), sw128_desc(smem_u32(sB2h) + 32 * s), idesc2, s > 0);
+                mma_f16(tmem + kTa, sw128_desc(smem_u32(sA2) + 32 * s), sw128_desc(smem_u32(sB2h) + 32 * s), idesc2, s > 0);
 #pragma unroll
             for (int s = 0; s < 4; ++s)
-                mma_f16(tmem + 64, sw128_desc(smem_u32(sA2) + 32 * s), sw128_desc(smem_u32(sB2l) + 32 * s), idesc2, 1);
+                mma_f16(tmem + kTa, sw128_desc(smem_u32(sA2) + 32 * s), sw128_desc(smem_u32(sB2l) + 32 * s), idesc2, 1);
             mma_commit(&mbar[1]);
         }
         if (!mbar_wait(&mbar[1], phase)) *sflag = 1;
@@ -494,7 +499,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : 2) k_sh_tc(const __gri
         float2 T[n];  // row k = lane of the first inverse stage (LGS)
         {
             uint32_t r[32];
-            GBWFS_TMEM_LD32(r, t_row + 64);
+            GBWFS_TMEM_LD32(r, t_row + kTa);
             tmem_wait_ld();
 #pragma unroll
             for (int d = 0; d < n; ++d) T[d] = make_float2(__uint_as_float(r[d]), __uint_as_float(r[16 + d]));
@@ -945,9 +950,9 @@ cudaError_t shape_tc_k(const ShArgs &a, LaunchShape *out) {
     if (e != cudaSuccess) return e;
     const int groups = (a.total + 3) / 4;
     const int cta_groups = (groups + WG - 1) / WG;
-    // resident CTAs per SM: two of two warpgroups or three of one (shared memory); their tensor
-    // memory (4 x 128 or 3 x 128 columns) always fits
-    const int per_sm = WG == 1 ? 3 : 2;
+    // resident CTAs per SM: one of six warpgroups, two of two or three of one (shared memory); their
+    // tensor memory (at most 512 columns) always fits
+    const int per_sm = WG == 1 ? 3 : WG == 2 ? 2 : 1;
     const int cap = a.grid_cap > 0 && a.grid_cap < 152 * per_sm ? a.grid_cap : 152 * per_sm;
     int blocks = cta_groups < cap ? cta_groups : cap;
     if (blocks < 1) blocks = 1;
@@ -969,9 +974,16 @@ cudaError_t shape_tc(const ShArgs &a, LaunchShape *out, bool f16) {
                    : shape_tc_k<n, N, nd, false, false, false, kWG, true>(a, out);
     if (a.mma_u)
         return f16 ? shape_tc_k<n, N, nd, false, true, true>(a, out) : shape_tc_k<n, N, nd, false, false, true>(a, out);
-    // ShArgs::cta_warps = 4: one warpgroup per CTA (else two)
+    // ShArgs::cta_warps = 4: one warpgroup per CTA, 24: six, 8: two.  Untuned launches (0) take six from
+    // kManyGroups groups on: a CTA of six shares one copy of the constant tiles and keeps 24 warps on
+    // an SM (uneven batch of 64, 28,900 groups in its largest class: 427 -> 405 us), but all of its
+    // warps start together, and a frame has too few groups to make up for it (ELT frame, 6,948 groups:
+    // 162 -> 165 us).
+    constexpr int kManyGroups = 16384;
     if (a.cta_warps == 4)
         return f16 ? shape_tc_k<n, N, nd, false, true, false, 1>(a, out) : shape_tc_k<n, N, nd, false, false, false, 1>(a, out);
+    if (a.cta_warps == 24 || (a.cta_warps == 0 && a.total >= 4 * kManyGroups))
+        return f16 ? shape_tc_k<n, N, nd, false, true, false, 6>(a, out) : shape_tc_k<n, N, nd, false, false, false, 6>(a, out);
     return f16 ? shape_tc_k<n, N, nd, false, true, false>(a, out) : shape_tc_k<n, N, nd, false, false, false>(a, out);
 }
 

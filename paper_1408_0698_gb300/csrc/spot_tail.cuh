@@ -84,15 +84,16 @@ __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 
-// K~ of subaperture v for this lane's frequency: the entries its share of the elongation stage takes
-// (rows past the band read the nearest row and are multiplied by zero).
+// K~ of a subaperture (column pairs first, so that a warp's read is contiguous) for this lane's
+// frequency: the entries its share of the elongation stage takes (rows past the band read the nearest
+// row and are multiplied by zero).
 template <int n>
 __device__ __forceinline__ void load_ktil(const float2 *kt, int lane, float4 (&kq)[n / 2]) {
     const int f = (int)(__brev((unsigned)lane) >> 27), dy = f < 16 ? f : f - 32;
     const int dyi = min(max(dy + n - 1, 0), 2 * n - 2);
-    const float4 *src = reinterpret_cast<const float4 *>(kt + dyi * n);  // n even: rows of 16-byte words
+    const float4 *src = reinterpret_cast<const float4 *>(kt) + dyi;
 #pragma unroll
-    for (int c = 0; c < n / 2; ++c) kq[c] = __ldg(src + c);
+    for (int c = 0; c < n / 2; ++c) kq[c] = __ldg(src + c * (2 * n - 1));
 }
 
 constexpr int kBScratch = 272;  // floats: the 16 x 16 image, its lower half 16 words off
