@@ -37,8 +37,12 @@
 // per-slice model (Sec. 4: one wavefront and one spot per sodium sub-layer, piled up with the
 // profile weights): the projection has made one OPD per slice (the layers through the slice's
 // cone); per slice the warp adds the slice's geometric term, forms U, and the warpgroup's
-// Y = U F^T runs on the tensor cores; the weighted |Y|^2 of the slices are summed in the warp's
-// shared rows, which then feed Ta = I Ga^T.
+// Y = U F^T runs on the tensor cores; the weighted |Y|^2 of the slices are summed in registers (row k in
+// lane k), then feed Ta = I Ga^T.  A slice's samples are loaded during the one before, and its field
+// and U are formed while the previous product runs.  Bound: latency (52 % issue, 58 % of the shared-memory
+// pipe at 16 warps per SM, 128 registers a thread).  ELT frame of 27,792 LGS subapertures with their
+// profiles: 332 us with the sums in shared memory and the slices one after the other -> 299 us, the same bits.
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <string.h>
@@ -62,27 +66,40 @@ constexpr uint32_t kTmemCols = 128 * kWG;  // per warpgroup: D1 columns [0, 64),
 // The field X of one subaperture in the warp's scratch as column pairs: entry [p][q/2] holds
 // (re q, re q+1, im q, im q+1) of row p (q even).  A lane forms whole entries (the pixels 2i, 2i + 1),
 // so that they are written as 16-byte words.  opd(i): the sample of pixel i; ref: the piston.
-template <int n, typename F>
-__device__ __forceinline__ void field_pairs(float4 *X4, F opd, float ref, float k_phase, const uint32_t *mk, int lane) {
-    constexpr int kE = n * n / 2, kM = (kE + 31) / 32;
+template <int n>
+struct FieldLane {  // a lane's pixel pairs
+    static constexpr int kE = n * n / 2, kM = (kE + 31) / 32;
     float o0[kM], o1[kM];
     uint32_t mw[kM];
+    static __device__ __forceinline__ int pair(int lane, int m) { return min(lane + 32 * m, kE - 1); }
+    __device__ __forceinline__ void load_mask(const uint32_t *mk, int lane) {
 #pragma unroll
-    for (int m = 0; m < kM; ++m) {  // all of the lane's loads first
-        const int i = min(lane + 32 * m, kE - 1);
-        o0[m] = opd(2 * i);
-        o1[m] = opd(2 * i + 1);
-        mw[m] = __ldg(mk + (i >> 4)) >> (2 * (i & 15));
+        for (int m = 0; m < kM; ++m) mw[m] = __ldg(mk + (pair(lane, m) >> 4)) >> (2 * (pair(lane, m) & 15));
     }
+    __device__ __forceinline__ void form(float4 *X4, float ref, float k_phase, int lane) const {
 #pragma unroll
-    for (int m = 0; m < kM; ++m) {
-        const int i = lane + 32 * m;
-        float s0, c0, s1, c1;
-        field_phasor(k_phase * (o0[m] - ref), s0, c0);
-        field_phasor(k_phase * (o1[m] - ref), s1, c1);
-        const bool l0 = mw[m] & 1u, l1 = mw[m] & 2u;
-        if (i < kE) X4[i] = make_float4(l0 ? c0 : 0.0f, l1 ? c1 : 0.0f, l0 ? s0 : 0.0f, l1 ? s1 : 0.0f);
+        for (int m = 0; m < kM; ++m) {
+            const int i = lane + 32 * m;
+            float s0, c0, s1, c1;
+            field_phasor(k_phase * (o0[m] - ref), s0, c0);
+            field_phasor(k_phase * (o1[m] - ref), s1, c1);
+            const bool l0 = mw[m] & 1u, l1 = mw[m] & 2u;
+            if (i < kE) X4[i] = make_float4(l0 ? c0 : 0.0f, l1 ? c1 : 0.0f, l0 ? s0 : 0.0f, l1 ? s1 : 0.0f);
+        }
     }
+};
+
+template <int n, typename F>
+__device__ __forceinline__ void field_pairs(float4 *X4, F opd, float ref, float k_phase, const uint32_t *mk, int lane) {
+    FieldLane<n> f;
+#pragma unroll
+    for (int m = 0; m < FieldLane<n>::kM; ++m) {  // all of the lane's loads first
+        const int i = f.pair(lane, m);
+        f.o0[m] = opd(2 * i);
+        f.o1[m] = opd(2 * i + 1);
+    }
+    f.load_mask(mk, lane);
+    f.form(X4, ref, k_phase, lane);
 }
 
 // U[q] = sum_p F[k][p] X[p][q] for this lane's DFT row k (lanes k >= N get zeros).  The rows k
@@ -161,9 +178,8 @@ struct TcLayout {
     static constexpr int oWarp = (oTab + tEnd * 8 + 15) / 16 * 16;  // per-warp scratch (float2)
     static constexpr int even(int x) { return (x + 1) & ~1; }
     // per warp: the field X (column pairs, 16-byte aligned); then an NGS's image rows (wI,
-    // [N][N + 1] floats) or the binned image (wB), over the consumed field, but for the per-slice
-    // variant, whose summed spot rows (wI) live across the slices' fields
-    static constexpr int wX = 0, wI = kSlices ? even(n * n) : 0, wB = wI;
+    // [N][N + 1] floats) or the binned image (wB), over the consumed field
+    static constexpr int wX = 0, wI = 0, wB = wI;
     static constexpr int i_end = wI + (N * (N + 1) + 1) / 2, b_end = wB + tail::kBScratch / 2;
     static constexpr int warp = even(n * n > (i_end > b_end ? i_end : b_end) ? n * n : (i_end > b_end ? i_end : b_end));
     static_assert(wB % 2 == 0, "16-byte aligned scratch");
@@ -574,8 +590,7 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : WG == 2 ? 2 : 1) k_sh_
 // The per-slice variant (see the file comment).
 template <int n, int nd, bool kF16>
 __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constant__ ShArgs a) {
-    constexpr bool kSlices = true;
-    using Lay = TcLayout<n, 32, nd, kSlices, false, kWG>;
+    using Lay = TcLayout<n, 32, nd, true, false, kWG>;
     using E = TcElt<kF16>;
     constexpr int N = 32, D2 = Lay::D2, nd2 = nd * nd;
     static_assert(6 * n <= 64 && n <= 16, "the split DFT operand must fit one 64-element K atom");
@@ -592,7 +607,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + Lay::oMisc + Lay::misc * wg);
     int *sflag = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 16);
     int *snext = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 20);  // next group (dynamic split)
-    int *snsl = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 32);   // slices per warp (kSlices)
+    int *snsl = reinterpret_cast<int *>(smem + Lay::oMisc + Lay::misc * wg + 32);   // slices per warp
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + Lay::oMisc + Lay::misc * kWG);
     const uint32_t bar_id = 1 + wg;
     auto wg_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(128) : "memory"); };
@@ -656,48 +671,79 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
         const InstDyn &D = a.dyn[W.inst];
         const int v = active ? g - W.subap_begin : 0;
         active = active && guard(v >= 0 && v < W.n_valid, a.status);
-        // slices: one for the elongation-kernel model; the warpgroup runs the largest count of
-        // its four subapertures (a subaperture with fewer adds nothing in the extra ones)
-        const SliceDesc *SD = (kSlices && active) ? W.slices : nullptr;
-        const int my_n = SD ? SD->n : 1;
-        int n_sl = 1;
-        if (kSlices) {
-            if (lane == 0) snsl[wq] = my_n;
-            wg_sync();
-            n_sl = max(max(snsl[0], snsl[1]), max(snsl[2], snsl[3]));
+        // slices (one for a natural star): the warpgroup runs the largest count of its four
+        // subapertures (a subaperture with fewer adds nothing in the extra ones)
+        const SliceDesc *SD = active ? W.slices : nullptr;
+        const int my_n = !active ? 0 : SD ? SD->n : 1;
+        if (lane == 0) snsl[wq] = my_n;
+        wg_sync();
+        const int n_sl = max(max(max(snsl[0], snsl[1]), max(snsl[2], snsl[3])), 1);
+        // the slice's OPD (projected through its cone) plus its geometric term
+        // k_s ((x - r_b).(r_b - r_L) + 1/2 |x - r_b|^2) about the subaperture centre r_b
+        const float *opd = D.opd + W.opd_off + (size_t)v * (n * n);
+        FieldLane<n> fl;
+        float geo0[fl.kM], geo1[fl.kM], ks = 0.0f, w_next = 0.0f;
+        if (active) {
+            float ebx = 0.0f, eby = 0.0f, dxp = 0.0f;
+            if (SD) {
+                const InstDesc &I = a.inst[W.inst];
+                const int id = __ldg(W.subap + v), sy = id / W.n_sub, sx = id - sy * W.n_sub;
+                const float half = 0.5f * (float)(W.n_sub * n - 1), c0 = 0.5f * (float)(n - 1);
+                dxp = (float)(W.pupil_dx_over_ds * I.ds);
+                ebx = ((float)(sx * n) + c0 - half) * dxp - (float)W.launch_x;
+                eby = ((float)(sy * n) + c0 - half) * dxp - (float)W.launch_y;
+            }
+            auto geo = [&](int i) -> float {
+                const int pp = i / n, qq = i - pp * n;
+                const float ux = ((float)qq - 0.5f * (float)(n - 1)) * dxp;
+                const float uy = ((float)pp - 0.5f * (float)(n - 1)) * dxp;
+                return fmaf(ux, ebx, fmaf(uy, eby, 0.5f * fmaf(ux, ux, uy * uy)));
+            };
+#pragma unroll
+            for (int m = 0; m < fl.kM; ++m) {
+                geo0[m] = geo(2 * fl.pair(lane, m));
+                geo1[m] = geo(2 * fl.pair(lane, m) + 1);
+            }
+            fl.load_mask(W.mask + (size_t)v * a.mask_words, lane);
         }
-        bool quit = false;
-        for (int sl = 0; sl < n_sl; ++sl) {
-            // field and U = F X (CUDA cores)
-            float2 U[n];
+        // a slice's samples, loaded ahead of their use
+        auto load_slice = [&](int sl) {
+            if (sl >= my_n) return;
+            const float *o = opd + (size_t)sl * a.slice_opd_stride;
+#pragma unroll
+            for (int m = 0; m < fl.kM; ++m) {
+                fl.o0[m] = __ldg(o + 2 * fl.pair(lane, m));
+                fl.o1[m] = __ldg(o + 2 * fl.pair(lane, m) + 1);
+            }
+            ks = SD ? SD->k[sl] : 0.0f;
+            w_next = SD ? SD->w[sl] : 1.0f;
+        };
+        // field and U = F X (CUDA cores); the field's last readers were the previous slice's field_rows
+        float2 U[n];
+        float w_sl = 0.0f;
+        auto slice_rows = [&](int sl) {
+            w_sl = sl < my_n ? w_next : 0.0f;
 #pragma unroll
             for (int q = 0; q < n; ++q) U[q] = make_float2(0.0f, 0.0f);
-            if (active && sl < my_n) {
-                // the slice's OPD (projected through its cone) plus its geometric term
-                // k_s ((x - r_b).(r_b - r_L) + 1/2 |x - r_b|^2) about the subaperture centre r_b
-                const float *opd = D.opd + W.opd_off + (size_t)sl * a.slice_opd_stride + (size_t)v * (n * n);
-                float ebx = 0.0f, eby = 0.0f, dxp = 0.0f, ks = 0.0f;
-                if (SD) {
-                    const InstDesc &I = a.inst[W.inst];
-                    const int id = __ldg(W.subap + v), sy = id / W.n_sub, sx = id - sy * W.n_sub;
-                    const float half = 0.5f * (float)(W.n_sub * n - 1), c0 = 0.5f * (float)(n - 1);
-                    dxp = (float)(W.pupil_dx_over_ds * I.ds);
-                    ebx = ((float)(sx * n) + c0 - half) * dxp - (float)W.launch_x;
-                    eby = ((float)(sy * n) + c0 - half) * dxp - (float)W.launch_y;
-                    ks = SD->k[sl];
-                }
-                auto geo = [&](int i) -> float {
-                    const int pp = i / n, qq = i - pp * n;
-                    const float ux = ((float)qq - 0.5f * (float)(n - 1)) * dxp;
-                    const float uy = ((float)pp - 0.5f * (float)(n - 1)) * dxp;
-                    return ks * fmaf(ux, ebx, fmaf(uy, eby, 0.5f * fmaf(ux, ux, uy * uy)));
-                };
-                const uint32_t *mk = W.mask + (size_t)v * a.mask_words;
-                const float ref = __ldg(opd) + geo(0);
-                field_pairs<n>(X4, [&](int i) { return __ldg(opd + i) + geo(i); }, ref, W.k_phase, mk, lane);
-                __syncwarp();
-                field_rows<n, N>(Fk, X4, lane, U);
+            if (sl >= my_n) return;
+            __syncwarp();
+#pragma unroll
+            for (int m = 0; m < fl.kM; ++m) {
+                fl.o0[m] = fmaf(ks, geo0[m], fl.o0[m]);
+                fl.o1[m] = fmaf(ks, geo1[m], fl.o1[m]);
             }
+            fl.form(X4, __shfl_sync(0xffffffffu, fl.o0[0], 0), W.k_phase, lane);
+            __syncwarp();
+            field_rows<n, N>(Fk, X4, lane, U);
+        };
+        load_slice(0);
+        slice_rows(0);
+        float Is[N];  // this row of the summed spot
+#pragma unroll
+        for (int m = 0; m < N; ++m) Is[m] = 0.0f;
+        bool quit = false;
+        for (int sl = 0; sl < n_sl; ++sl) {
+            load_slice(sl + 1);
             // FP16: U times 2^eu (exact), eu from the slice's largest component
             int eu = 0;
             if constexpr (kF16) {
@@ -745,77 +791,52 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
                     mma_f16(tmem, sw128_desc(smem_u32(sA1) + 32 * s), sw128_desc(smem_u32(sB1) + 32 * s), idesc1, s > 0);
                 mma_commit(&mbar[0]);
             }
-            // the elongation-kernel model completes mbar[0] once per group like mbar[1]
-            if (!mbar_wait(&mbar[0], kSlices ? phase0 : phase)) *sflag = 1;
-            if (kSlices) phase0 ^= 1u;
+            // the next slice's rows while the product runs
+            const float wsl = w_sl;
+            const float uy = kF16 ? pow2f(-eu) : 1.0f;  // FP16: Y carries 2^eu
+            if (sl + 1 < n_sl) slice_rows(sl + 1);
+            __syncwarp();
+            if (!mbar_wait(&mbar[0], phase0)) *sflag = 1;
+            phase0 ^= 1u;
             fence_after_sync();
-            // Y row from TMEM -> I = |Y|^2; the elongation-kernel model writes the second operand
-            // row [I_hi | I_lo] at once, the per-slice model adds w_s I into the warp's rows
-            {
-                float *dstI = (active && D.st_I && (!kSlices || sl == n_sl - 1))
-                                  ? D.st_I + W.int_off + (size_t)v * (N * N) + lane * N
-                                  : nullptr;
-                const float wsl = (SD && sl < my_n) ? SD->w[sl] : (kSlices && sl > 0 ? 0.0f : 1.0f);
-                const float uy = kF16 ? pow2f(-eu) : 1.0f;  // FP16: Y carries 2^eu
+            // Y row from TMEM -> I = |Y|^2, weighted into the row's sum
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t r[16], r2[16];
-                    GBWFS_TMEM_LD16(r, t_row + 16 * hh);
-                    GBWFS_TMEM_LD16(r2, t_row + 32 + 16 * hh);
-                    tmem_wait_ld();
-                    float I[16];
+            for (int hh = 0; hh < 2; ++hh) {
+                uint32_t r[16], r2[16];
+                GBWFS_TMEM_LD16(r, t_row + 16 * hh);
+                GBWFS_TMEM_LD16(r2, t_row + 32 + 16 * hh);
+                tmem_wait_ld();
 #pragma unroll
-                    for (int m = 0; m < 16; m += 2) {  // column pairs: each half as fmaf(yr, yr, yi * yi)
-                        const float2 yr = make_float2(__uint_as_float(r[m]), __uint_as_float(r[m + 1]));
-                        const float2 yi = make_float2(__uint_as_float(r2[m]), __uint_as_float(r2[m + 1]));
-                        const float2 y2 = __ffma2_rn(yr, yr, __fmul2_rn(yi, yi));
-                        const float2 iv = kF16 ? __fmul2_rn(__fmul2_rn(y2, make_float2(uy, uy)), make_float2(uy, uy)) : y2;
-                        I[m] = iv.x;
-                        I[m + 1] = iv.y;
-                    }
-                    if (kSlices) {
-                        float *ir = Iw + lane * (N + 1) + 16 * hh;
-#pragma unroll
-                        for (int m = 0; m < 16; ++m) {
-                            const float tot = sl == 0 ? wsl * I[m] : fmaf(wsl, I[m], ir[m]);
-                            ir[m] = tot;
-                            if (dstI) dstI[16 * hh + m] = tot;
-                        }
-                        continue;
-                    }
-                    if (dstI) {
-#pragma unroll
-                        for (int m = 0; m < 16; ++m) dstI[16 * hh + m] = I[m];
-                    }
-                    if (active && !W.is_lgs) {
-#pragma unroll
-                        for (int m = 0; m < 16; ++m) Iw[lane * (N + 1) + 16 * hh + m] = I[m];
-                    }
-#pragma unroll
-                    for (int c2 = 0; c2 < 2; ++c2) {
-                        uint32_t hw[4], lw[4];
-#pragma unroll
-                        for (int e2 = 0; e2 < 4; ++e2) {
-                            E::split2(I[c2 * 8 + 2 * e2], I[c2 * 8 + 2 * e2 + 1], hw[e2], lw[e2]);
-                        }
-                        *reinterpret_cast<uint4 *>(sA2 + sw128_off(row, (2 * hh + c2) * 8)) =
-                            make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                        *reinterpret_cast<uint4 *>(sA2 + sw128_off(row, (4 + 2 * hh + c2) * 8)) =
-                            make_uint4(lw[0], lw[1], lw[2], lw[3]);
-                    }
+                for (int m = 0; m < 16; m += 2) {  // column pairs: each half as fmaf(yr, yr, yi * yi)
+                    const float2 yr = make_float2(__uint_as_float(r[m]), __uint_as_float(r[m + 1]));
+                    const float2 yi = make_float2(__uint_as_float(r2[m]), __uint_as_float(r2[m + 1]));
+                    const float2 y2 = __ffma2_rn(yr, yr, __fmul2_rn(yi, yi));
+                    const float2 iv = kF16 ? __fmul2_rn(__fmul2_rn(y2, make_float2(uy, uy)), make_float2(uy, uy)) : y2;
+                    const float2 acc = __ffma2_rn(make_float2(wsl, wsl), iv, make_float2(Is[16 * hh + m], Is[16 * hh + m + 1]));
+                    Is[16 * hh + m] = acc.x;
+                    Is[16 * hh + m + 1] = acc.y;
                 }
             }
             fence_before_sync();  // these TMEM reads precede the next slice's MMA
-            __syncwarp();         // the warp's rows are complete before the next slice adds to them
         }
         if (quit) break;
+        if (active && D.st_I) {
+            float *dstI = D.st_I + W.int_off + (size_t)v * (N * N) + lane * N;
+#pragma unroll
+            for (int m = 0; m < N; ++m) dstI[m] = Is[m];
+        }
+        if (active && !W.is_lgs) {
+            __syncwarp();  // the field's readers are done: the rows alias it
+#pragma unroll
+            for (int m = 0; m < N; ++m) Iw[lane * (N + 1) + m] = Is[m];
+        }
         int ei = 0;  // FP16: the second operand carries 2^ei
-        if (kSlices) {
+        {
             // the summed rows -> second operand row [I_hi | I_lo] (after the last slice's MMA)
             if constexpr (kF16) {
                 float mx = 0.0f;
 #pragma unroll
-                for (int c = 0; c < N; ++c) mx = fmaxf(mx, Iw[lane * (N + 1) + c]);
+                for (int c = 0; c < N; ++c) mx = fmaxf(mx, Is[c]);
                 ei = f16_scale_exp(warp_max(mx));
             }
             const float si = kF16 ? pow2f(ei) : 1.0f;
@@ -824,7 +845,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_sh_tc_sl(const __grid_constan
                 uint32_t hw[4], lw[4];
 #pragma unroll
                 for (int e2 = 0; e2 < 4; ++e2) {
-                    const float i0 = Iw[lane * (N + 1) + c4 * 8 + 2 * e2], i1 = Iw[lane * (N + 1) + c4 * 8 + 2 * e2 + 1];
+                    const float i0 = Is[c4 * 8 + 2 * e2], i1 = Is[c4 * 8 + 2 * e2 + 1];
                     E::split2(kF16 ? i0 * si : i0, kF16 ? i1 * si : i1, hw[e2], lw[e2]);
                 }
                 *reinterpret_cast<uint4 *>(sA2 + sw128_off(row, c4 * 8)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
