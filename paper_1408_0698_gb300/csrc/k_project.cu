@@ -438,6 +438,10 @@ cudaError_t launch_project(const ProjArgs &a, ProjRange blocks, cudaStream_t s, 
     LaunchShape sh;
     cudaError_t e = project_launch_shape(a, blocks, &sh);
     if (e != cudaSuccess) return e;
+    // beside the uplink kernel's few CTAs, whose FP64 sums the launch ends up waiting for: whole CTAs of
+    // blocks rather than a block on every SM (two LGS of 22 x 22, n = 10, four layers, uplink on: 36.9 us
+    // spread, 30.7 us packed; 33.5 and 33.1 us for 7 x 7, n = 16)
+    if (after_uplink) sh.grid.x = std::min(sh.grid.x, (unsigned)(blocks.full + blocks.part + kProjWarps - 1) / kProjWarps);
     ProjArgs b = a;
     b.n_full = blocks.full;
     b.n_blocks = blocks.full + blocks.part;
