@@ -643,6 +643,33 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         if (e != cudaSuccess) return cuda_fail(h, e, "uplink launch");
         if ((e = cudaEventRecord(h->ev_uplink, stream)) != cudaSuccess) return cuda_fail(h, e, "uplink event");
     }
+    // the per-slice model on kernels that read projected slices: one projection of every (WFS, slice)
+    // pair of the group into the slice OPDs, then the kernel's per-slice variant
+    auto slices_group = [&](const SpotGroup &G, cudaStream_t ls) -> wfs_status {
+        if (G.total == 0) return WFS_OK;
+        pa.wfs = G.d_sl_wfs;
+        pa.n_wfs = G.sl_count;
+        pa.block_base = pa.part_base = 0;
+        pa.work = h->d_work + 2 * (h->groups.size() + 1) + 2 * (&G - h->groups.data());
+        pa.dyn[0].opd = h->d_opd_sl;
+        long slot = timed_begin(h, "project", ls);
+        cudaError_t err = launch_project(pa, G.sl_blocks, ls, ls == stream && h->n_uplink > 0 && !h->timing);
+        timed_end(h, slot, ls);
+        pa.dyn[0].opd = dyn.opd;
+        if (err != cudaSuccess) return cuda_fail(h, err, "projection launch");
+        const bool copies = st && st->opd;  // the OPD stage: the first slice's OPDs
+        for (int q = 0; copies && q < G.count; ++q) {
+            const WfsDesc &d = h->wfs_host[G.first + q];
+            if ((err = cudaMemcpyAsync(st->opd + d.opd_off, h->d_opd_sl + d.opd_off,
+                                       sizeof(float) * (size_t)d.n_valid * d.n * d.n, cudaMemcpyDeviceToDevice, ls)) !=
+                cudaSuccess)
+                return cuda_fail(h, err, "OPD stage copy");
+        }
+        if ((err = launch_group(G, ls, !copies, 0, (long long)h->opd_total)) != cudaSuccess)
+            return cuda_fail(h, err, "spot launch");
+        return WFS_OK;
+    };
+    wfs_status sts;
     size_t k = 0;
     for (size_t j = 0; j < h->groups.size(); ++j) {
         const SpotGroup &G = h->groups[j];
@@ -657,39 +684,22 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         // a small FP32 group (a few NGS subapertures) or a 64-point one projects inside its spot
         // kernel: one launch that starts with the call and owns its SMs only while it runs
         const wfs_geometry &geo = h->geoms[G.geom].g;
-        const bool fused = G.kind == kSpotGeneric || G.per_slice || (is_tc(G.kind) && geo.n_fft == 64) ||
+        const bool fused = G.kind == kSpotGeneric || (is_tc(G.kind) && geo.n_fft == 64) ||
                            (G.kind == kSpotRow && !(geo.n_fft == 32 && geo.n_det == 16));
-        if (!fused && (e = project(G, ss)) != cudaSuccess) return cuda_fail(h, e, "projection launch");
-        if ((e = launch_group(G, ss, !fused, fused ? 1 : 0)) != cudaSuccess)
-            return cuda_fail(h, e, "spot launch");
+        if (G.per_slice && G.sl_projected) {
+            if ((sts = slices_group(G, ss)) != WFS_OK) return sts;
+        } else {
+            if (!fused && (e = project(G, ss)) != cudaSuccess) return cuda_fail(h, e, "projection launch");
+            if ((e = launch_group(G, ss, !fused, fused ? 1 : 0)) != cudaSuccess)
+                return cuda_fail(h, e, "spot launch");
+        }
         if ((e = cudaEventRecord(h->ev_join[k], ss)) != cudaSuccess) return cuda_fail(h, e, "join");
         ++k;
     }
     if (!h->groups.empty()) {
         const SpotGroup &G = h->groups[big];
         if (G.per_slice && G.sl_projected) {
-            // the per-slice model: one projection of every (WFS, slice) pair into the slice OPDs,
-            // then the 32-point kernel's per-slice variant
-            pa.wfs = G.d_sl_wfs;
-            pa.n_wfs = G.sl_count;
-            pa.block_base = pa.part_base = 0;
-            pa.work = h->d_work + 2 * (h->groups.size() + 1) + 2 * big;
-            pa.dyn[0].opd = h->d_opd_sl;
-            long slot = timed_begin(h, "project", stream);
-            e = launch_project(pa, G.sl_blocks, stream, h->n_uplink > 0 && !h->timing);
-            timed_end(h, slot, stream);
-            pa.dyn[0].opd = dyn.opd;
-            if (e != cudaSuccess) return cuda_fail(h, e, "projection launch");
-            const bool copies = st && st->opd;  // the OPD stage: the first slice's OPDs
-            for (int q = 0; copies && q < G.count; ++q) {
-                const WfsDesc &d = h->wfs_host[G.first + q];
-                if ((e = cudaMemcpyAsync(st->opd + d.opd_off, h->d_opd_sl + d.opd_off,
-                                         sizeof(float) * (size_t)d.n_valid * d.n * d.n, cudaMemcpyDeviceToDevice,
-                                         stream)) != cudaSuccess)
-                    return cuda_fail(h, e, "OPD stage copy");
-            }
-            if (G.total > 0 && (e = launch_group(G, stream, !copies, 0, (long long)h->opd_total)) != cudaSuccess)
-                return cuda_fail(h, e, "spot launch");
+            if ((sts = slices_group(G, stream)) != WFS_OK) return sts;
         } else if (G.per_slice) {
             // the per-slice model projects one wavefront per sodium slice inside the spot kernel
             if (G.total > 0 && (e = launch_group(G, stream, false, 2)) != cudaSuccess)

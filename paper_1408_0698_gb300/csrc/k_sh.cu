@@ -328,6 +328,8 @@ cudaError_t tc_launch_shape(const ShArgs &a, LaunchShape *out, bool f16);
 cudaError_t tc64_launch_shape(const ShArgs &a, LaunchShape *out, bool f16);
 
 cudaError_t spot_launch_shape(int kind, const ShArgs &a, LaunchShape *out) {
+    // the 32-point tensor-core kernels read projected samples only
+    if (a.project != 0 && is_tc(kind) && a.N != 64) return cudaErrorInvalidValue;
     switch (kind) {
         case kSpotGeneric: return generic_shape(a, out);
         case kSpotRow: return row_launch_shape(a, out);
