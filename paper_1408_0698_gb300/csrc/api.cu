@@ -681,11 +681,15 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
         for (int q = 0; q < G.count; ++q) needs_uplink |= h->wfs_host[G.first + q].uplink != nullptr;
         if (needs_uplink && (e = cudaStreamWaitEvent(ss, h->ev_uplink, 0)) != cudaSuccess)
             return cuda_fail(h, e, "uplink wait");
-        // a small FP32 group (a few NGS subapertures) or a 64-point one projects inside its spot
-        // kernel: one launch that starts with the call and owns its SMs only while it runs
+        // A group of the generic kernel or a 64-point one (a few NGS subapertures) projects inside its
+        // spot kernel: one launch that starts with the call and owns its SMs only while it runs.  The
+        // kernel with a warp per subaperture takes a projection launch before it: a lane gathers its
+        // samples of every layer one after the other, and the SMs that such a launch kept to itself are
+        // missed by the large group.  Frame with 6 LGS of 80 x 80 and ten layers, side group of 20 x 20
+        // n = 8: 137.0 us self-projected, 119.3 apart; 3 LGS + 1 NGS of 40 x 40, three layers, side group
+        // of 36 x 36 n = 6: 41.3 and 28.9 us; of 28 to 80 subapertures, within 3 us either way.
         const wfs_geometry &geo = h->geoms[G.geom].g;
-        const bool fused = G.kind == kSpotGeneric || (is_tc(G.kind) && geo.n_fft == 64) ||
-                           (G.kind == kSpotRow && !(geo.n_fft == 32 && geo.n_det == 16));
+        const bool fused = G.kind == kSpotGeneric || (is_tc(G.kind) && geo.n_fft == 64);
         if (G.per_slice && G.sl_projected) {
             if ((sts = slices_group(G, ss)) != WFS_OK) return sts;
         } else {

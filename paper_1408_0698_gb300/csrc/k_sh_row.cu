@@ -530,7 +530,6 @@ __global__ void __launch_bounds__(256, n <= 10 ? 3 : 2) k_sh_row(const __grid_co
 namespace {
 
 constexpr int kRowMaxSmem = 200 * 1024;
-constexpr int kRowSelfProjectSmem = 160 * 1024;
 
 template <int n, int cN = 0, int cnd = 0>
 cudaError_t row_shape(const ShArgs &a, LaunchShape *out) {
@@ -561,9 +560,7 @@ cudaError_t row_shape(const ShArgs &a, LaunchShape *out) {
         const int spread = (a.total + 2 * 152 - 1) / (2 * 152);
         warps = spread < 8 ? (spread < 1 ? 1 : spread) : 8;
     }
-    int smem = row_smem(n, a.N, a.nd, warps, a.project != 0).total;
-    // self-projecting on a side stream: no projection CTA may share the SM (k_sh.cu)
-    if (a.project == 1 && smem < kRowSelfProjectSmem) smem = kRowSelfProjectSmem;
+    const int smem = row_smem(n, a.N, a.nd, warps, a.project != 0).total;
     int per_sm = 65536 / (((r + 7) & ~7) * 32 * warps);
     per_sm = min(per_sm, 227 * 1024 / (smem + 1024));
     per_sm = max(1, min(per_sm, 64 / warps));

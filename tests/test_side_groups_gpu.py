@@ -59,3 +59,31 @@ def test_per_slice_side_group(side, precision, big, uplink):
     _check_wfs(cfg, scr, 0.013, together, sel=sel)
     w.close()
     v.close()
+
+
+@pytest.mark.parametrize("n_sub,n,N,nd,precision,lgs,layers", [
+    (20, 8, 16, 8, inputs.PREC_BF16X3, False, 1), (36, 6, 24, 12, inputs.PREC_FP16S, False, 3),
+    (36, 6, 24, 12, inputs.PREC_BF16X3, True, 10), (10, 10, 32, 16, inputs.PREC_FP32, True, 3),
+    (7, 16, 32, 32, inputs.PREC_FP32, False, 2), (3, 9, 21, 7, inputs.PREC_FP32, True, 10)])
+def test_fp32_side_group_has_its_projection(n_sub, n, N, nd, precision, lgs, layers):
+    """A side group of the warp-per-subaperture kernel, below and above the largest group's limits for
+    projecting in the spot kernel: a projection launch of its own, the same bits as alone."""
+    base = inputs.config2(inputs.PREC_BF16X3)
+    ar = np.arange(layers, dtype=np.float64)
+    lay = dataclasses.replace(base.layers, alt_m=1000.0 * ar, wind_vx_mps=3.0 + ar, wind_vy_mps=-5.0 * ar, x0_m=0.3 * ar,
+                              y0_m=-0.2 * ar, weights=np.full(layers, 1.0 / layers))
+    star = dataclasses.replace(base.stars[0 if lgs else 3], geometry_index=1)
+    cfg = dataclasses.replace(base, layers=lay, geometries=base.geometries + [inputs.Geometry(n_sub, n, N, nd, 0.5, precision)],
+                              stars=base.stars + [star])
+    scr = torch.as_tensor(inputs.make_screens(lay, 3)).cuda()
+    w, v = native.Wfs(cfg, seed=2), native.Wfs(_alone(cfg), seed=2)
+    a, b = (torch.zeros((x.total, 2), device="cuda") for x in (w, v))
+    native.wfs_measure(w.h, scr.data_ptr(), 0.021, a.data_ptr(), 0)
+    native.wfs_measure(v.h, scr.data_ptr(), 0.021, b.data_ptr(), 0)
+    native.wfs_timing_enable(w.h, True)
+    native.wfs_measure(w.h, scr.data_ptr(), 0.021, a.data_ptr(), 0)
+    torch.cuda.synchronize()
+    assert native.wfs_timing_read(w.h)["project"][0] == 2
+    assert torch.equal(a[-v.total:], b) and bool(torch.any(b != 0))
+    w.close()
+    v.close()
