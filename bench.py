@@ -157,7 +157,7 @@ def source_sha(names):
 
 
 KERNEL_SOURCES = {"spot": ["k_sh.cu", "noise.cuh", "proj_math.cuh", "internal.h"],
-                  "spot_row": ["k_sh_row.cu", "self_project.cuh", "proj_math.cuh", "spot_tail.cuh", "noise.cuh", "internal.h"],
+                  "spot_row": ["k_sh_row.cuh", "k_sh_row.cu", "k_sh_row_slices.cu", "self_project.cuh", "proj_math.cuh", "spot_tail.cuh", "noise.cuh", "internal.h"],
                   "spot_tc": ["k_sh_tc.cu", "spot_tail.cuh", "noise.cuh", "internal.h", "tcgen05.cuh"],
                   "spot_tc64": ["k_sh_tc64.cu", "noise.cuh", "proj_math.cuh", "internal.h", "tcgen05.cuh"],
                   "noise_cog": ["k_noise_cog.cu", "spot_tail.cuh", "noise.cuh", "internal.h"],
