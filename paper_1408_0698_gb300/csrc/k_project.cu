@@ -4,8 +4,8 @@
 //
 // A warp owns a block: up to 64 consecutive pupil columns of a run of subapertures by up to 11 pupil
 // rows of one subaperture row; lane i takes the columns i and i + 32.  Per layer, the box of screen
-// pixels that the block's taps touch (at most 68 x 12) is copied to the warp's own ring of three slots
-// by cp.async, two layers ahead of the interpolation; nothing but the warp itself waits for it, so the
+// pixels that the block's taps touch (at most 68 x 12) is copied to one of the warp's own two slots by
+// cp.async, a layer ahead of the interpolation; nothing but the warp itself waits for it, so the
 // warps of an SM run out of step and cover each other's copies.  The geometry of all of a block's
 // boxes is formed at its start, a layer per lane.  Going down a column, pupil row p + 1 falls on the
 // same screen row pair as row p or one row lower (the cone factor is at most one for a tiled WFS), so
@@ -75,11 +75,6 @@ __device__ __forceinline__ int wrap_once(int i, int S) {
     return i - (i >= S ? S : 0);
 }
 
-__device__ __forceinline__ int wrap_any(int i, int S) {
-    const int r = i % S;
-    return r < 0 ? r + S : r;
-}
-
 __device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -139,24 +134,51 @@ __device__ __forceinline__ void rows_unit(float2 (&acc)[kBlockRows], const float
 }
 
 // The copy of a box across the periodic screen's edges (word by word) or of rows without 16-byte
-// alignment (element by element).  Out of line: few boxes take it, and the kernel's code stays short.
+// alignment (element by element: every box of a screen whose side is no multiple of 4 or whose address is
+// off).  A lane keeps its columns, wrapped once, and goes down the rows.  Out of line: the kernel's code
+// stays short for the boxes that are copied as they lie.  ELT frame, screens one float off 16 bytes:
+// 110.8 us with a division and two remainders per element -> 48.8 us (35.7 us for aligned screens); with
+// boxes across the edges 39.6 -> 37.0 us.
 __device__ __noinline__ void copy_box_slow(const LayerBox *b, uint32_t dst, int S, int lane) {
     const float *scr = b->scr;
-    const int cs = b->cs, rs = b->rs;
+    const int cs = b->cs, n_rows = b->rows;
+    auto column = [&](int c) {  // cs + c wrapped; cs < S, c < kBoxCols
+        c += cs;
+        while (c >= S) c -= S;
+        return c;
+    };
+    int row = b->rs;  // in [0, S)
     if (b->mode == kEdge) {
-        const int w4 = b->cols >> 2, n_words = b->rows * w4;
-        for (int idx = lane; idx < n_words; idx += 32) {
-            const int r = idx / w4, w = idx - r * w4;
-            copy16(dst + r * kPitch + 16 * w, scr + (size_t)wrap_any(rs + r, S) * S + wrap_any(cs + 4 * w, S));
+        const int w4 = b->cols >> 2, word = lane & 15;
+        const int c = column(4 * word);
+        const bool on = word < w4;
+        row += lane >> 4;
+        for (int r = lane >> 4; r < n_rows; r += 2, row += 2) {  // half a warp per row
+            while (row >= S) row -= S;
+            if (on) copy16(dst + r * kPitch + 16 * word, scr + (size_t)row * S + c);
+        }
+        // the words past the sixteenth, one or two a row
+        const int more = w4 - 16;
+        if (lane < n_rows * more) {
+            const int r = more == 2 ? lane >> 1 : lane, w = 16 + (more == 2 ? lane & 1 : 0);
+            row = b->rs + r;
+            while (row >= S) row -= S;
+            copy16(dst + r * kPitch + 16 * w, scr + (size_t)row * S + column(4 * w));
         }
     } else {
-        const int w = b->cols, n_el = b->rows * w;
-        for (int idx = lane; idx < n_el; idx += 32) {
-            const int r = idx / w, c = idx - r * w;
-            copy4(dst + r * kPitch + 4 * c, scr + (size_t)wrap_any(rs + r, S) * S + wrap_any(cs + c, S));
+        const int c0 = column(lane), c1 = column(lane + 32), c2 = column(lane + 64);
+        const bool on0 = lane < b->cols, on1 = lane + 32 < b->cols, on2 = lane + 64 < b->cols;
+        for (int r = 0; r < n_rows; ++r) {
+            const float *src = scr + (size_t)row * S;
+            const uint32_t d = dst + r * kPitch + 4 * lane;
+            if (on0) copy4(d, src + c0);
+            if (on1) copy4(d + 128, src + c1);
+            if (on2) copy4(d + 256, src + c2);
+            row = row + 1 == S ? 0 : row + 1;
         }
     }
 }
+static_assert(kBoxCols <= 72 && 2 * (kBlockRows + 2) <= 32, "at most two words past the sixteenth, a lane each");
 
 // A warp's block seg (of W.segs) of a tiled WFS.
 __device__ __forceinline__ void project_block(const ProjArgs &a, const ProjSmem &L, const WfsDesc &W, const InstDesc &I,
