@@ -550,11 +550,11 @@ __global__ void __launch_bounds__(128 * WG, WG == 1 ? 3 : WG == 2 ? 2 : 1) k_sh_
                         Ui[c] = tail::mul2(Ti[c], sg);
                     }
                     tail::lgs_binned<n, nd>(Ur, Ui, fft[(s ? 10 : 5) * 32 + lane], Bw, fft, a.Gc, kq, lane, Bv);
-                    tail::finish<nd>(Bv, W, D, v, lane, false, slopes + (s ? a.pair_off : 0));
+                    tail::centroid<nd>(Bv, W, v, lane, slopes + (s ? a.pair_off : 0));
                 }
             } else {
                 tail::ngs_binned<nd>(Iw, lane, Bv);
-                tail::finish<nd>(Bv, W, D, v, lane, false, slopes);
+                tail::centroid<nd>(Bv, W, v, lane, slopes);
                 if (lane == 0) {
                     slopes[a.pair_off + 2 * v] = -slopes[2 * v];
                     slopes[a.pair_off + 2 * v + 1] = -slopes[2 * v + 1];

@@ -436,5 +436,35 @@ __device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc 
     }
 }
 
+// The centroid of a binned image without noise and without stage outputs (the push-pull pairs), from the
+// differences of pixels mirrored about the centre: d = B[iy][ix] - B[iy][nd-1-ix] and e likewise down the
+// columns, so that the sums' roundings are those of the small differences and not of the pixels: the two
+// slopes of a pair share what comes before, and would not average it out as two measurements do.  RMS
+// error against 64 bits, FP16S, 80 x 80, n = 10: 3.79e-6 of the rows' RMS for two measurements, 3.82e-6 for
+// a pair by finish()'s sums, 3.02e-6 by these; 64 modes of it (BF16X3) 1,236 -> 1,191 us.
+template <int nd>
+__device__ __forceinline__ void centroid(const float (&Bv)[nd / 2], const WfsDesc &W, int v, int lane, float *slopes) {
+    constexpr int J = nd / 2;
+    static_assert(nd == 16, "columns mirror within 16 lanes, rows across the half-warps");
+    const int ix = lane & 15, half = lane >> 4;
+    const float cd = 0.5f * (float)(nd - 1);
+    float sc = 0.0f, sx = 0.0f, sy = 0.0f;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        sc += Bv[j];
+        sx += Bv[j] - __shfl_xor_sync(0xffffffffu, Bv[j], 15);
+        sy = fmaf((float)(half * J + j) - cd, Bv[j] - __shfl_xor_sync(0xffffffffu, Bv[J - 1 - j], 16), sy);
+    }
+    // every pair is counted from both of its ends
+    sx = 0.5f * warp_sum(((float)ix - cd) * sx);
+    sc = warp_sum(sc);
+    sy = 0.5f * warp_sum(sy);
+    if (lane == 0) {
+        const bool ok = sc > 0.0f && W.photons * __ldg(W.fill + v) > 0.0f;
+        slopes[2 * v] = ok ? sx / sc : 0.0f;
+        slopes[2 * v + 1] = ok ? sy / sc : 0.0f;
+    }
+}
+
 }  // namespace tail
 }  // namespace gbwfs
