@@ -103,20 +103,24 @@ def spot_flops(n, N, nd, lgs, kernel=""):
     return f
 
 
+#: The sizes (n, N, nd) compiled into the warp-per-subaperture FP32 kernel.
+ROW_SIZES = [(8, 16, 8), (6, 24, 12), (8, 32, 16), (10, 32, 16)]
+
+
 def row_flops(n, N, nd, lgs):
     """FP32 flops (FMA = 2) of one subaperture in the warp-per-subaperture FP32 kernel, whose centred
     DFTs are folded about their centres (h = ceil(n/2) mirrored inputs, half of the outputs computed,
     each giving its mirror by one more complex add): U 4Nhn + 4Nn; the fold of U 4Nh; Y per row and
-    column pair 8h + 4 adds, two |.|^2 of 3; LGS: T 2 adds and 4n per column pair (half of the 4n
-    where N is a multiple of 4, after 6 more adds per two pairs), its fold 4Nn, A 8 per (dy, dx) and
-    row pair and 4 adds, M 12 for each of +-dy and 4 adds, Q 8 per (dy, dx) and row pair and 4 adds,
-    B 4 per (dx, iy) and column pair and 2 adds; NGS: binning N^2.  Photometry and centroid 6 nd^2."""
+    column pair 8h + 4 adds, two |.|^2 of 3; LGS: T 2 adds and 4n per column pair (compiled sizes: 8 adds
+    and 4n per two column pairs), its fold 4n per row pair, A 8 per (dy, dx) and row pair and 4 adds, M 6
+    for each of +-dy and 4 adds, Q 8 per (dy, dx) and row pair and 4 adds, B 4 per (dx, iy) and column
+    pair and 4 adds; NGS: binning N^2.  Photometry and centroid 6 nd^2."""
     h, hN, hd = (n + 1) // 2, (N + 1) // 2, (nd + 1) // 2
     f = 4 * N * h * n + 4 * N * n + 4 * N * h + N * hN * (8 * h + 4 + 6)
     if not lgs:
         return f + N * N + 6 * nd * nd
-    f += N * (hN // 2) * (4 + 6 + 4 * n) if N % 4 == 0 else N * hN * (2 + 4 * n)
-    f += 4 * N * n + n * n * (8 * hN + 4 + 24 + 4) + hd * n * (8 * n + 4) + nd * hd * (4 * n + 2)
+    f += N * (hN // 2) * (8 + 4 * n) if (n, N, nd) in ROW_SIZES else N * hN * (2 + 4 * n)
+    f += 4 * hN * n + n * n * (8 * hN + 4 + 12 + 4) + hd * n * (8 * n + 4) + nd * hd * (4 * n + 4)
     return f + 6 * nd * nd
 
 
