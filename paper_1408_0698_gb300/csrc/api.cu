@@ -1859,7 +1859,9 @@ std::string class_key(const BatchClass &c, int total) {
     std::string name = p.name;
     for (char &ch : name)
         if (ch == ' ') ch = '_';
-    return "kind" + std::to_string(c.kind) + "_n" + std::to_string(c.geom->g.n_pix_sub) + "_N" +
+    // a kind of its own name for the FP32 kernel with a warp per subaperture: "kind1" lines were tuned for
+    // the kernel of N = 32 that had the number before
+    return (c.kind == kSpotRow ? "row" : "kind" + std::to_string(c.kind)) + "_n" + std::to_string(c.geom->g.n_pix_sub) + "_N" +
            std::to_string(c.geom->g.n_fft) + "_nd" + std::to_string(c.geom->g.n_det) + "_sub" +
            std::to_string(bucket) + "_" + name;
 }
