@@ -724,9 +724,13 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
     return WFS_OK;
 }
 
+// Mirrors of the handle's loop.
+int loop_mirrors(wfs_handle h) { return h->loop ? (int)h->loop->dms.size() : 0; }
+
 // Slice tables of every LGS (weights, curvatures, per-layer cones including any mirror layers),
-// uploaded to h->d_slices.
-wfs_status refresh_slices(wfs_handle h) {
+// uploaded to h->d_slices.  n_dm: the mirrors among the layers.  A slice so low under a layer that its
+// footprint there would not fit the screen is refused: the samples are wrapped once.
+wfs_status refresh_slices(wfs_handle h, int n_dm) {
     if (!h->per_slice) return WFS_OK;
     std::vector<SliceDesc> sd(h->gs.size());
     memset(sd.data(), 0, sizeof(SliceDesc) * sd.size());
@@ -740,8 +744,11 @@ wfs_status refresh_slices(wfs_handle h) {
         for (int s = 0; s < d.n; ++s) {
             d.w[s] = (float)G.na_w[s];
             d.k[s] = (float)(1.0 / G.gs.range_m - 1.0 / G.na_alt[s]);
-            for (int l = 0; l < kMaxProjLayers; ++l) {
+            for (int l = 0; l < h->inst_host.n_layers + n_dm; ++l) {
                 const double c = (1.0 - h->inst_host.alt[l] / G.na_alt[s]) * r;
+                if (0.5 * geo.n_sub * geo.n_pix_sub * std::fabs(c) + 2.0 >= h->S)
+                    return fail(h, WFS_EINVAL, "guide star " + std::to_string(g) + ": a sodium slice's footprint on layer " +
+                                                   std::to_string(l) + " is larger than the screen");
                 d.c[s][l].x = (float)c;
                 d.c[s][l].y = (float)(c - (double)d.c[s][l].x);
             }
@@ -753,8 +760,10 @@ wfs_status refresh_slices(wfs_handle h) {
 
 // 32-point kernels read per-slice OPDs made by one projection launch over copies of the WFS
 // entries whose range is the slice altitude (the cone) and whose OPD goes to slice s; the copies
-// follow the work table (rebuilt when it changes, e.g. the uplink switch).
-wfs_status build_slice_projection(wfs_handle h) {
+// follow the work table (rebuilt when it changes, e.g. the uplink switch).  n_dm: the mirrors among
+// the layers.  A slice below a layer sees it mirrored (a negative cone), which a projection block's
+// boxes do not describe: such a pair is projected by direct gathers.
+wfs_status build_slice_projection(wfs_handle h, int n_dm) {
     cudaError_t e;
     for (SpotGroup &G : h->groups) {
         cudaFree(G.d_sl_wfs);
@@ -769,6 +778,8 @@ wfs_status build_slice_projection(wfs_handle h) {
             for (size_t sl = 0; sl < ns; ++sl) {
                 WfsDesc d = d0;
                 if (d0.is_lgs) d.range_m = gd.na_alt[sl];
+                for (int l = 0; d0.is_lgs && l < h->inst_host.n_layers + n_dm; ++l)
+                    if (h->inst_host.alt[l] > d.range_m) d.tiled = 0;
                 d.opd_off = d0.opd_off + (long long)(sl * h->opd_total);
                 place_blocks(d, blocks);
                 t.push_back(d);
@@ -2321,9 +2332,11 @@ wfs_status wfs_loop_create(wfs_handle h, int n_dm, const wfs_dm *dms, const floa
     }
     if ((e = cudaMemcpy(h->d_inst, &h->inst_host, sizeof(InstDesc), cudaMemcpyHostToDevice)) != cudaSuccess)
         return bail(e, "layer table");
-    if (refresh_slices(h) != WFS_OK) {
+    wfs_status st = refresh_slices(h, n_dm);
+    if (st == WFS_OK && h->per_slice) st = build_slice_projection(h, n_dm);
+    if (st != WFS_OK) {
         loop_free(lp);
-        return WFS_ECUDA;
+        return st;
     }
     h->loop = lp;
     *out = lp;
@@ -2518,7 +2531,7 @@ wfs_status wfs_set_uplink(wfs_handle h, int gs, double diameter_m, int samples) 
     if (on != (g.up_diam > 0)) h->n_uplink += on ? 1 : -1;
     g.up_diam = on ? diameter_m : 0.0;
     g.up_n = on ? samples : 0;
-    if (h->per_slice) return build_slice_projection(h);  // the slice copies carry the uplink too
+    if (h->per_slice) return build_slice_projection(h, loop_mirrors(h));  // the slice copies carry the uplink too
     return WFS_OK;
 }
 
@@ -2564,9 +2577,9 @@ wfs_status wfs_set_lgs_model(wfs_handle h, int per_slice) {
         }
     }
     h->per_slice = per_slice != 0;
-    if (per_slice && refresh_slices(h) != WFS_OK) {
+    if (const wfs_status st = refresh_slices(h, loop_mirrors(h)); st != WFS_OK) {
         h->per_slice = false;
-        return WFS_ECUDA;
+        return st;
     }
     for (SpotGroup &G : h->groups) {
         bool lgs = false;
@@ -2597,7 +2610,7 @@ wfs_status wfs_set_lgs_model(wfs_handle h, int per_slice) {
         }
         G.sl_projected = per_slice && (is_tc(G.kind) || G.kind == kSpotRow);
     }
-    if (build_slice_projection(h) != WFS_OK) return WFS_ECUDA;
+    if (build_slice_projection(h, loop_mirrors(h)) != WFS_OK) return WFS_ECUDA;
     if ((e = cudaMemcpy(h->d_wfs, h->wfs_host.data(), sizeof(WfsDesc) * h->wfs_host.size(), cudaMemcpyHostToDevice)) !=
         cudaSuccess)
         return cuda_fail(h, e, "work table");
