@@ -71,12 +71,13 @@ struct SpotGroup {
     int kind = 0;            // SpotKind
     int grid_cap = 0, cta_warps = 0;
     ProjRange proj_base{0, 0}, proj_count{0, 0};  // this group's projection blocks
-    // LGS per-slice model: the group runs a per-slice spot kernel (the 32-point kernels' variants
-    // after a projection of every (WFS, slice) pair, else the self-projecting generic kernel); the
-    // kind and launch shape of the elongation-kernel model are kept to restore it
+    // LGS per-slice model: the group runs a per-slice spot kernel (the variants of the tensor-core and
+    // the warp-per-subaperture kernel after a projection of every (WFS, slice) pair, else the
+    // self-projecting generic kernel); the kind and launch shape of the elongation-kernel model are
+    // kept to restore it
     bool per_slice = false;
     int base_kind = 0, base_grid_cap = 0, base_cta_warps = 0;
-    // 32-point kernels: the per-slice OPDs come from one projection of every (WFS, slice) pair
+    // the per-slice OPDs come from one projection of every (WFS, slice) pair
     bool sl_projected = false;
     WfsDesc *d_sl_wfs = nullptr;
     int sl_count = 0;
@@ -601,7 +602,7 @@ wfs_status measure_impl(wfs_handle h, const float *screens, double t, float *slo
     static thread_local ShArgs sa;
     // project_mode: 0 = a projection launch precedes, 1 = self-projecting on a side stream,
     // 2 = self-projecting on the caller's stream
-    // slice_stride > 0: the per-slice 32-point kernels read slice s of the OPDs from d_opd_sl
+    // slice_stride > 0: the per-slice kernels read slice s of the OPDs from d_opd_sl
     auto launch_group = [&](const SpotGroup &G, cudaStream_t ls, bool after_project, int project_mode,
                             long long slice_stride = 0) -> cudaError_t {
         memset(&sa, 0, offsetof(ShArgs, dyn));
@@ -758,7 +759,7 @@ wfs_status refresh_slices(wfs_handle h, int n_dm) {
     return e == cudaSuccess ? WFS_OK : cuda_fail(h, e, "slice tables");
 }
 
-// 32-point kernels read per-slice OPDs made by one projection launch over copies of the WFS
+// The per-slice kernels read OPDs made by one projection launch over copies of the WFS
 // entries whose range is the slice altitude (the cone) and whose OPD goes to slice s; the copies
 // follow the work table (rebuilt when it changes, e.g. the uplink switch).  n_dm: the mirrors among
 // the layers.  A slice below a layer sees it mirrored (a negative cone), which a projection block's

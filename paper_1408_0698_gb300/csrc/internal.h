@@ -130,7 +130,7 @@ struct ShArgs {
     int grid_cap;        // maximum CTAs (0 = the launcher's default)
     int cta_warps;       // warps per CTA where the kernel allows a choice (0 = default)
     int n_inst;
-    // Dynamic work split of the 32-point kernels: {next ticket, CTAs done}, zero between
+    // Dynamic work split of the kernels that own a subaperture per warp: {next ticket, CTAs done}, zero between
     // launches (the last CTA to finish resets it), used by one launch at a time; null = a
     // static split.
     int *work;
@@ -144,7 +144,7 @@ struct ShArgs {
     // 32-point tensor-core kernels, push-pull pairs: the slopes of the negated wavefront too, pair_off
     // floats after those of the wavefront (no noise, no stage outputs); 0 = off
     long long pair_off;
-    int split_noise;     // 32-point kernels: 1 = store the expected image (dyn.st_E, required)
+    int split_noise;     // 32-point tensor-core kernels: 1 = store the expected image (dyn.st_E, required)
                          // and stop; launch_noise_cog completes the measurement; 0 = no instance
                          // has noise on: the centroid of the expected image in the spot kernel
     InstDyn dyn[kMaxInstances];

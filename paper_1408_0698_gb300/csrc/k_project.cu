@@ -12,17 +12,19 @@
 // a row's lower interpolated tap pair is the next row's upper pair; the two columns travel as packed
 // FP32x2 operations.
 //
-// A WFS whose pupil samples the screens more coarsely than one screen pixel, and every WFS of the
-// allocation-free entry point, is projected by direct gathers (proj_direct.cuh), 32 blocks of 2 x 2
-// pixels a warp.  Every form does the same per-tap arithmetic in the same order: the same OPD.
+// A WFS whose pupil samples the screens more coarsely than one screen pixel, a sodium slice below a
+// layer, and every WFS of the allocation-free entry point, is projected by direct gathers
+// (proj_direct.cuh), 32 blocks of 2 x 2 pixels a warp.  Every form does the same per-tap arithmetic in
+// the same order: the same OPD.
 //
-// Bound: issue and latency (45 % issue at 16 warps per SM), and at the start of a launch the instruction
+// Bound: issue and latency (48 % issue at 15 warps per SM), and at the start of a launch the instruction
 // fetches and the dependent loads of the first blocks: the rare copies are kept out of line for that
 // (with them inlined, 45 -> 49 us).  Measured against boxes of up to 400 columns moved by bulk copies of
-// two producer warps to eight consumer warps of a CTA (library events, L2 flushed): ELT frame 44.6 -> 42
-// us, 48 (LGS, slice) pairs of it 235 -> 209 us, 316 subapertures on one layer 15.0 -> 12.5 us, 64
-// measurements on one layer 96.5 -> 101 us; an uneven batch of 64 frames 477 -> 430 us.  Three slots,
-// 24 warps per SM, and preparing a block while the one before it runs gained nothing.
+// two producer warps to eight consumer warps of a CTA (library events, L2 flushed): ELT frame 44.6 -> 37
+// us, 48 (LGS, slice) pairs of it 235 -> 207 us, 316 subapertures on one layer 15.0 -> 12.5 us; an uneven
+// batch of 64 frames 477 -> 430 us.  Slower: 64 measurements on one layer 96.5 -> 102 us (nothing to copy
+// ahead), 3 sensors of 37 x 37, n = 9, on five layers 15.4 -> 16.7 us.  Three slots, 24 warps per SM, and
+// preparing a block while the one before it runs gained nothing.
 #include <algorithm>
 #include <mutex>
 

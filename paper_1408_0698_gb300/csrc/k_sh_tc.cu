@@ -19,8 +19,9 @@
 // in the 128-byte-swizzled K-major layout (8-row x 128-byte atoms); one elected
 // thread issues the MMAs and commits them to an mbarrier; every wait is bounded
 // and a timeout is reported in the status word (the kernel then frees its tensor
-// memory and returns).  U = F X, the column transform, binning, photometry,
-// noise and the centroid run on the CUDA cores exactly as in the FP32 kernels.
+// memory and returns).  U = F X, the elongation stages, binning, photometry and,
+// without noise, the centroid run on the CUDA cores (spot_tail.cuh); the noise
+// has a pass of its own (k_noise_cog.cu).
 //
 // Bound: the shared-memory and load/store wavefronts with their latency (61 % of that pipe, 46 % issue at
 // 16 warps per SM; with 20 or 24 warps the same time, so it is the pipe).  G of the binning stage comes
@@ -31,7 +32,12 @@
 // rows of n put a lane's word into a sector of its own: 86.3 us.
 //
 // CTA = two warpgroups (4 warps each), or six in launches of many subapertures (shape_tc); warp w of a
-// warpgroup owns subaperture 4g + w of its group g and its lane k owns DFT row k, which is also TMEM lane 32 w + k of both accumulators.
+// warpgroup owns subaperture 4g + w of its group g and its lane k owns DFT row k, which is also TMEM lane
+// 32 w + k of both accumulators.
+//
+// The pair variant (kPair, ShArgs::pair_off) takes the slopes of a wavefront and of its negative from one
+// pass: the negative's spot is the spot mirrored, so only the tail runs again (tail::lgs_binned,
+// tail::centroid).  Chunk of 64 modes of an 80 x 80 LGS: 1,001 us (two measurements of 32 modes: 857 us).
 //
 // The per-slice variant (k_sh_tc_sl, launched with ShArgs::slice_opd_stride) runs the LGS
 // per-slice model (Sec. 4: one wavefront and one spot per sodium sub-layer, piled up with the

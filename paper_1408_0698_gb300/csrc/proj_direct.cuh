@@ -2,9 +2,9 @@
 // layers' screens, shifted for the star's direction and the wind and shrunk by the LGS cone,
 // summed by bilinear interpolation): one thread per 2x2 block of pupil pixels, every tap read
 // from the screens in global memory.  Used where the pupil samples the screens more coarsely than
-// one screen pixel (no shared-memory tile pays) and by the allocation-free entry point.  The
-// per-tap arithmetic and its order are those of the tiled forms, so every form gives the same
-// OPD bit for bit.
+// one screen pixel (no shared-memory tile pays), for sodium slices below a layer (a box has no
+// negative cone) and by the allocation-free entry point.  The per-tap arithmetic and its order are
+// those of the tiled forms, so every form gives the same OPD bit for bit.
 #pragma once
 #include "internal.h"
 #include "proj_math.cuh"

@@ -1,7 +1,8 @@
-// spot_tail.cuh -- the stages of the 32-point spot kernels that follow the first
+// spot_tail.cuh -- the stages of the 32-point tensor-core spot kernels that follow the first
 // transfer-domain stage, on the CUDA cores, for one subaperture owned by one warp
 // (Sec. 4 LGS SH: elongation by the sodium kernel, binning, noise-added image,
-// centroid).  Shared by the FP32 and tensor-core kernels.
+// centroid), and the noise pass's noise and centroid.  The FP32 kernel with a warp per
+// subaperture takes the small helpers only (packed arithmetic, warp sums).
 //
 //   M[dy][dx] = Kt[dy][dx] sum_k Ga(dy, k) T[k][dx]       (k = lane: a 32-point DFT)
 //   Q[iy][dx] = sum_dy G(dy, iy) M[dy][dx]                 (an nd-point DFT over dy)
@@ -402,10 +403,10 @@ __device__ __forceinline__ void noise_centroid(const float (&ev)[nd / 2], const 
 }
 
 // Photometry, then the centroid of the expected image in place (a measurement without noise); with
-// split, the expected image is stored and the noise kernel completes the measurement.  slopes: the WFS's.  The sums of
-// the centroid run in noise_centroid's order.  Without noise the image would only travel to the
-// noise kernel and back: ELT frame, FP32, 125.5 us + 17.2 us for that pass -> 129.4 us in place
-// (the frame 181.5 -> 172.7 us); a calibration's chunk of 64 measurements 857 + 148 us -> 869 us.
+// split, the expected image is stored and the noise kernel completes the measurement.  slopes: the
+// WFS's.  The sums of the centroid run in noise_centroid's order.  Without noise the image would only
+// travel to the noise kernel and back: 16 us of a noise-free ELT frame; a calibration's chunk of 64
+// measurements 857 + 148 us -> 869 us in place.
 template <int nd>
 __device__ __forceinline__ void finish(const float (&Bv)[nd / 2], const WfsDesc &W, const InstDyn &D, int v,
                                        int lane, bool split, float *slopes) {
