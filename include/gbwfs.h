@@ -299,7 +299,7 @@ wfs_status wfs_batch_measure_subset(wfs_batch b, int slot, int n_active, const i
                                     float *const *slopes_out, void *stream);
 /*
  * Autotuner: times the candidate launch shapes of every kernel class on these inputs
- * (persistent grid size; warps per CTA for the FP32 32-point kernel), keeps the
+ * (persistent grid size; warps per CTA for the FP32 and tensor-core kernels), keeps the
  * fastest for later calls, and appends it to the file named by the environment
  * variable GBWFS_TUNE_CACHE (if set), from which wfs_batch_create reads earlier
  * choices.  Synchronises `stream`; leaves the slopes of one measurement in slopes_out.
