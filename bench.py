@@ -62,9 +62,9 @@ def q_dft_flops(n, nd):
 
 def dft_forms(kernel, N):
     """How a spot kernel computes the dense DFT stages: U = F X with the rows k and k + N/2 paired
-    ("r2": F[k + N/2][p] = F[k][p] (-1)^p i^(n-1)) in the tensor-core kernels up to N = 32 and in
-    the FP32 32-point kernel, which also takes Y = U F^T and Ta = I Ga^T by column quadruples
-    (m + 8j: "r4"); otherwise dense."""
+    ("r2": F[k + N/2][p] = F[k][p] (-1)^p i^(n-1)) in the tensor-core kernels up to N = 32; otherwise
+    dense.  "spot_n32" names an earlier FP32 kernel, which also took Y = U F^T and Ta = I Ga^T by column
+    quadruples (m + 8j: "r4"); today's is counted by row_flops."""
     if kernel.startswith("spot_n32"):
         return {"U": "r2", "Y": "r4", "Ta": "r4"}
     if kernel.startswith("spot_tc") and not kernel.startswith("spot_tcu") and N <= 32:
